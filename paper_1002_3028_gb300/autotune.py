@@ -28,6 +28,7 @@ CACHE = os.path.join(_build.BUILD, "autotune.json")
 # double the tiles of small lattices.  A batch spreads each step over many lattices and
 # profits from longer bands.
 LATTICE_CANDIDATES: Tuple[Tuple[int, int, int], ...] = (
+    (64, 0, 1), (32, 0, 1),  # band 0: the library's own choice, which keeps small lattices on the chip
     (64, 1, 1), (64, 2, 1), (64, 3, 1), (64, 4, 1), (64, 5, 1), (64, 6, 1), (64, 7, 1), (64, 8, 1), (64, 9, 1),
     (64, 10, 1), (64, 6, 2), (32, 1, 1), (32, 2, 1), (32, 4, 1), (32, 6, 1), (32, 8, 1),
 )

@@ -266,6 +266,10 @@ Layout make_layout(const lbm_desc *d)
 
 struct lbm_batch;
 
+struct ResPlan {  // tiles of a lattice kept on the chip (res_plan)
+    int shape, ns, nb, warps;
+};
+
 struct lbm_lattice {
     lbm_desc d;
     lbm_batch *batch;  // the batch this lattice belongs to, if any
@@ -292,6 +296,14 @@ struct lbm_lattice {
     int64_t sync_items;
     unsigned sync_cbase, sync_fbase;
     bool sync_captured;    // a launch was captured into a graph: reset before every launch
+    ResPlan res;           // resident launch (lbm_resident.cuh): its tiles; shape -1: none
+    // the tiles' inboxes of the resident launch, allocated by its first
+    // launch: valid for tiles laid out as res_key (0 = reset before the next launch), with
+    // res_base the number of the next launch's first step
+    void *res_box;
+    size_t res_bytes;
+    int64_t res_key;
+    unsigned res_base;
 
     void *buf(int b) const { return mem + L.off_buf[b]; }
     template <class T> T *at(size_t off) const { return reinterpret_cast<T *>(mem + off); }
@@ -387,6 +399,8 @@ lbm::StepParams<float> params_f(const lbm_lattice *h)
 // warp tiles per work item of lbm_step: the set value, else 1
 int item_group(const lbm_lattice *h) { return h->group > 0 ? h->group : 1; }
 
+void res_plan(lbm_lattice *h);
+
 // Launch shape of the step kernel: a persistent grid of one-warp CTAs (by
 // default) working through strip x band tiles.  A tile of step t + 1 waits
 // for the tiles around it of step t, which precede it by one step's worth
@@ -440,6 +454,153 @@ int plan_launch(lbm_lattice *h)
     const int64_t ntiles = (int64_t)nstrips * ((h->d.nr + h->band_eff - 1) / h->band_eff);
     h->ctas_max = per_sm * std::max(1, h->sms);
     h->ctas = (int)std::min<int64_t>(h->ctas_max, (ntiles + h->warps - 1) / h->warps);
+    res_plan(h);
+    return LBM_OK;
+}
+
+// Lattices that fit the chip run their steps there (lbm_resident.cuh): strips of 64 columns
+// (FP64 32), cut into tiles of one CTA each, every CTA resident.  Of the tile shapes, in FP32
+// arithmetic: eight rows, one a warp, while one tile a SM is enough (us per step: 200 x 96
+// FP32 3.8 with tiles of 8 rows, 4.2 of 6, 4.5 of 4, 6.1 of 16 rows with two rows a warp);
+// then the same with two CTAs a SM, whose registers leave room for six warps each
+// (640 x 160 FP16 moment-split 6.4 in tiles of 5 and 6 rows, 7.4 of 14 with two rows a warp);
+// then sixteen rows, two a warp, two CTAs a SM (1024 x 256 FP32 7.4).  FP64 is bound by its
+// arithmetic: the tiles that spread it over the SMs best.  The step kernel takes 8.8, 15.8
+// and 12.4 us on the three lattices and keeps those that do not fit, those with periodic
+// ends or in the AA layout, and those whose launch shape the caller has set.
+cudaError_t res_occupancy(const lbm_lattice *h, int shape, int warps, int *per_sm)
+{
+    switch (h->d.storage) {
+    case LBM_F64: return lbm::occupancy_res_f64(shape, warps, per_sm);
+    case LBM_F32: return lbm::occupancy_res_f32(shape, warps, per_sm);
+    case LBM_F16: return lbm::occupancy_res_f16(shape, warps, per_sm);
+    case LBM_F16S: return lbm::occupancy_res_f16s(shape, warps, per_sm);
+    case LBM_BF16S: return lbm::occupancy_res_bf16s(shape, warps, per_sm);
+    default: return lbm::occupancy_res_bf16(shape, warps, per_sm);
+    }
+}
+
+void res_plan(lbm_lattice *h)
+{
+    const lbm_desc &d = h->d;
+    h->res.shape = -1;
+    if (h->aa || d.bc_in == LBM_IN_PERIODIC || h->band > 0 || h->group > 0 || h->warps != 1 ||
+        h->nv != default_nv(d.storage))
+        return;
+    auto fits = [&](int shape, int nb) {
+        const int W = strip_cols(d.storage);
+        const int ns = (d.nx + W - 1) / W;
+        const int rows = (d.nr + nb - 1) / nb;
+        if (nb < 1 || rows > lbm::res_rows(shape) || (nb > 1 && d.nr / nb < 2) || (ns > 1 && d.nx / ns < 2))
+            return false;
+        const int warps = (rows + lbm::res_rpw(shape) - 1) / lbm::res_rpw(shape);
+        int per_sm = 0;
+        if (res_occupancy(h, shape, warps, &per_sm) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if ((int64_t)ns * nb > (int64_t)per_sm * h->sms)
+            return false;
+        h->res = ResPlan{shape, ns, nb, warps};
+        return true;
+    };
+    // tiles up when `slots` CTAs share the lattice in tiles of at least `rows` rows
+    auto up = [&](int cols, int slots, int rows) {
+        return std::min(slots / ((d.nx + cols - 1) / cols), (d.nr + rows - 1) / rows);
+    };
+    const int cols = strip_cols(d.storage), one = h->sms, two = 2 * h->sms;
+    if (d.storage == LBM_F64)
+        (void)(fits(0, up(cols, one, 4)) || fits(0, up(cols, two, 4)) || fits(2, up(cols, one, 4)));
+    else
+        (void)(fits(0, up(cols, one, 8)) || fits(0, up(cols, two, 4)) || fits(1, up(cols, two, 4)));
+}
+
+cudaError_t res_launch(lbm_lattice *h, const lbm::ResCtl &ctl, const ResPlan &r, cudaStream_t s)
+{
+    switch (h->d.storage) {
+    case LBM_F64: return lbm::launch_res_f64(params_d(h), ctl, r.shape, r.warps, s);
+    case LBM_F32: return lbm::launch_res_f32(params_f(h), ctl, r.shape, r.warps, s);
+    case LBM_F16: return lbm::launch_res_f16(params_f(h), ctl, r.shape, r.warps, s);
+    case LBM_F16S: return lbm::launch_res_f16s(params_f(h), ctl, r.shape, r.warps, s);
+    case LBM_BF16S: return lbm::launch_res_bf16s(params_f(h), ctl, r.shape, r.warps, s);
+    default: return lbm::launch_res_bf16(params_f(h), ctl, r.shape, r.warps, s);
+    }
+}
+
+lbm::ResCtl res_ctl(const lbm_lattice *h, const ResPlan &r, int nsteps)
+{
+    lbm::ResCtl ctl;
+    ctl.box = static_cast<unsigned long long *>(h->res_box);
+    ctl.base = h->res_base;
+    ctl.nsteps = nsteps;
+    ctl.ns = r.ns;
+    ctl.nb = r.nb;
+    ctl.spin_limit = lbm::RUN_SPIN_LIMIT;
+    ctl.first = 0;
+    return ctl;
+}
+
+// The inboxes of the plan's tiles, ready for a launch on s.  *ok = false: there is no memory
+// for them, or none yet on a stream that is being captured.
+int res_ready(lbm_lattice *h, const ResPlan &r, bool capturing, cudaStream_t s, bool *ok)
+{
+    const size_t bytes = (size_t)16 * (size_t)r.ns * (size_t)r.nb *
+                         (size_t)lbm::res_box_words(h->d.storage == LBM_F64 ? 8 : 4, r.shape);
+    const int64_t key = ((int64_t)(r.shape + 1) << 40) | ((int64_t)r.ns << 20) | r.nb;
+    *ok = r.ns * r.nb == 1;
+    if (*ok)
+        return LBM_OK;
+    cudaError_t e = cudaSuccess;
+    if (h->res_bytes < bytes) {
+        if (capturing)
+            return LBM_OK;
+        if (h->res_box)
+            cudaFreeAsync(h->res_box, s);
+        h->res_box = nullptr;
+        h->res_bytes = 0;
+        h->res_key = 0;
+        if (cudaMallocAsync(&h->res_box, bytes, s) != cudaSuccess) {
+            cudaGetLastError();
+            h->res_box = nullptr;
+            return LBM_OK;
+        }
+        h->res_bytes = bytes;
+    }
+    if (h->res_key != key || h->sync_captured) {
+        e = cudaMemsetAsync(h->res_box, 0, bytes, s);
+        h->res_key = e == cudaSuccess ? key : 0;
+        h->res_base = 0;
+        if (e != cudaSuccess)
+            return cuda_fail(e, "inbox reset");
+    }
+    *ok = true;
+    return LBM_OK;
+}
+
+constexpr int kResMinSteps = 2;  // one step reads and writes the lattice once either way
+
+// *done: steps taken (fewer than nsteps when the tiles cannot all be resident after all)
+int res_step(lbm_lattice *h, const ResPlan &r, int nsteps, bool capturing, cudaStream_t s, int *done)
+{
+    bool ok = false;
+    *done = 0;
+    int rc = res_ready(h, r, capturing, s, &ok);
+    if (rc || !ok)
+        return rc;
+    cudaError_t e = res_launch(h, res_ctl(h, r, nsteps), r, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return LBM_OK;
+    }
+    if (e != cudaSuccess) {
+        h->res_key = 0;
+        return cuda_fail(e, "resident step kernel launch");
+    }
+    h->res_base += (unsigned)nsteps;
+    h->cur ^= (nsteps & 1);
+    h->step += nsteps;
+    h->prev_valid = true;
+    *done = nsteps;
     return LBM_OK;
 }
 
@@ -932,6 +1093,11 @@ int lbm_create(const lbm_desc *d, void *dev_mem, size_t bytes, lbm_lattice **out
     h->sync_items = 0;
     h->sync_cbase = h->sync_fbase = 0;
     h->sync_captured = false;
+    h->res.shape = -1;
+    h->res_box = nullptr;
+    h->res_bytes = 0;
+    h->res_key = 0;
+    h->res_base = 0;
     cudaGetDevice(&h->device);
     h->sms = 1;
     cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
@@ -1015,6 +1181,10 @@ void lbm_destroy(lbm_lattice *h)
         // released in stream order after the lattice's last use: no host synchronisation
         cudaStreamWaitEvent(nullptr, h->last, 0);
         cudaFreeAsync(h->mem, nullptr);
+    }
+    if (h->res_box) {
+        cudaStreamWaitEvent(nullptr, h->last, 0);
+        cudaFreeAsync(h->res_box, nullptr);
     }
     h->mem = nullptr;
     cudaEventDestroy(h->ready);
@@ -1103,6 +1273,21 @@ static int step_impl(lbm_lattice *h, int32_t nsteps, lbm_stream stream)
         }
         return LBM_OK;
     }
+    // The counters of either launch carry on from the previous launch (RunCtl, ResCtl) unless
+    // the tiles changed, a wait ran out (lbm_check) or the launch goes into a graph,
+    // whose replays must each start from a reset.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess)
+        return cuda_fail(cudaGetLastError(), "querying the stream");
+    if (cap != cudaStreamCaptureStatusNone)
+        h->sync_captured = true;
+    if (nsteps >= kResMinSteps && h->res.shape >= 0) {
+        int done = 0;
+        const int rc = res_step(h, h->res, nsteps, cap != cudaStreamCaptureStatusNone, s, &done);
+        if (rc)
+            return rc;
+        nsteps -= done;
+    }
     const int nstrips = (d.nx + 32 * h->nv - 1) / (32 * h->nv);
     const int64_t items = (int64_t)lbm::item_cols(nstrips, ctl.group) * ((d.nr + h->band_eff - 1) / h->band_eff);
     // steps per launch: the work indices of one launch stay below 2^31
@@ -1113,14 +1298,6 @@ static int step_impl(lbm_lattice *h, int32_t nsteps, lbm_stream stream)
     ctl.radius = h->band_eff >= 2 ? 1 : 2;
     ctl.wrap = d.bc_in == LBM_IN_PERIODIC ? 1 : 0;
     ctl.spin_limit = lbm::RUN_SPIN_LIMIT;
-    // The counters carry on from the previous launch (RunCtl) unless the item
-    // count changed, a wait ran out (lbm_check) or the launch goes into a graph,
-    // whose replays must each start from a reset.
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess)
-        return cuda_fail(cudaGetLastError(), "querying the stream");
-    if (cap != cudaStreamCaptureStatusNone)
-        h->sync_captured = true;
     for (int64_t done = 0; done < nsteps;) {
         const int m = (int)std::min<int64_t>(per_launch, nsteps - done);
         cudaError_t e = cudaSuccess;
@@ -1241,7 +1418,26 @@ int lbm_selftest_wait_timeout(lbm_lattice *h, int32_t *flags)
     }
     if (e != cudaSuccess)
         return cuda_fail(e, "self-test launch");
-    return lbm_check(h, flags);  // synchronises, reads and clears the status
+    rc = lbm_check(h, flags);  // synchronises, reads and clears the status
+    const ResPlan r = h->res;
+    if (rc || r.shape < 0 || r.ns * r.nb < 2)
+        return rc;
+    // the resident launch: every tile starts at its second step and waits for first steps
+    // that never run
+    bool ok = false;
+    rc = res_ready(h, r, false, s, &ok);
+    if (rc || !ok)
+        return rc;
+    lbm::ResCtl res = res_ctl(h, r, 2);
+    res.spin_limit = 64;
+    res.first = 1;
+    e = res_launch(h, res, r, s);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "self-test launch");
+    int32_t second = 0;
+    rc = lbm_check(h, &second);
+    *flags &= second;  // LBM_STATUS_TIMEOUT only if both launches' waits gave up
+    return rc;
 }
 
 int lbm_set_item_group(lbm_lattice *h, int32_t group)
@@ -1249,6 +1445,7 @@ int lbm_set_item_group(lbm_lattice *h, int32_t group)
     if (!valid(h) || group < 0 || group > 64)
         return fail(LBM_ERR_INVALID_ARG, "bad handle or group (0..64)");
     h->group = group;
+    res_plan(h);
     return LBM_OK;
 }
 
@@ -1297,7 +1494,7 @@ int lbm_check(lbm_lattice *h, int32_t *flags)
     if (e != cudaSuccess)
         return cuda_fail(e, "reading the status word");
     if (v & lbm::STATUS_TIMEOUT)
-        h->sync_items = 0;  // a launch stopped early: its counters are not where the host expects
+        h->sync_items = h->res_key = 0;  // a launch stopped early: its counters are not where the host expects
     *flags = v;
     return LBM_OK;
 }

@@ -7,6 +7,7 @@
 
 #include "lbm.h"
 #include "lbm_aa_batch.cuh"
+#include "lbm_resident.cuh"
 
 namespace lbm {
 
@@ -21,6 +22,9 @@ namespace lbm {
                                    const RunCtl &ctl, int warps_per_cta, int ctas, int far, int nv,   \
                                    cudaStream_t s);                                                    \
     cudaError_t occupancy_batch_##TAG(int warps_per_cta, int nv, int *ctas_per_sm);                    \
+    cudaError_t launch_res_##TAG(const StepParams<C> &p, const ResCtl &ctl, int shape, int warps,          \
+                                 cudaStream_t s);                                                      \
+    cudaError_t occupancy_res_##TAG(int shape, int warps, int *ctas_per_sm);                           \
     cudaError_t launch_fields_##TAG(const StepParams<C> &p, void *out, int out_f64, cudaStream_t s);   \
     cudaError_t launch_fill_##TAG(const StepParams<C> &p, cudaStream_t s);                             \
     cudaError_t launch_diag_##TAG(const StepParams<C> &p, int have_prev, double *partials, int nblocks,     \
@@ -50,6 +54,9 @@ namespace lbm {
                                    const RunCtl &ctl, int warps_per_cta, int ctas, int far, int nv,   \
                                    cudaStream_t s);                                                    \
     cudaError_t occupancy_batch_##TAG(int warps_per_cta, int nv, int *ctas_per_sm);                    \
+    cudaError_t launch_res_##TAG(const StepParams<C> &p, const ResCtl &ctl, int shape, int warps,          \
+                                 cudaStream_t s);                                                      \
+    cudaError_t occupancy_res_##TAG(int shape, int warps, int *ctas_per_sm);                           \
     cudaError_t launch_fields_##TAG(const StepParams<C> &p, void *out, int out_f64, cudaStream_t s);   \
     cudaError_t launch_fill_##TAG(const StepParams<C> &p, cudaStream_t s);                             \
     cudaError_t launch_diag_##TAG(const StepParams<C> &p, int have_prev, double *partials, int nblocks,     \

@@ -209,15 +209,27 @@ __device__ __forceinline__ C lin_part(const StepParams<C> &p, int q, C jx, C jr,
     return C(0.25) * dT + (p.T0 + dT) * p.hir0 * edot<C>(ex4(q - 9), ey4(q - 9), jx, jr);
 }
 
+// A population from its stored deviation d and the moments stored with it (the linear part
+// added), and the deviation of a population v at moments (jx, jr, dT) (the linear part taken
+// off), with the roundings of stage_pops and of collide_row's store: for the kernels whose
+// values must have the step kernel's bits without its surroundings (rn_*: below).
+template <class C> __device__ __forceinline__ C split_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d);
+template <class C> __device__ __forceinline__ C split_sub(const StepParams<C> &p, int q, C jx, C jr, C dT, C v);
+// The same with the roundings of write_ghosts: an edge node's populations from what it
+// stored, and what its ghost cells store.
+template <class C> __device__ __forceinline__ C edge_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d);
+template <class C> __device__ __forceinline__ C edge_sub(const StepParams<C> &p, int q, C jx, C jr, C dT, C v);
+
 // Moments a ghost cell (ci, cj) carries when node (i, j), with moments
 // (jx, jr, dT), writes it: the one node whose rule fills an axis, open-top,
 // inlet, outflow or periodic ghost cell writes its own moments there
-// (mirrored across the axis; the prescribed inflow at the inlet).  The
+// (mirrored across the axis; the prescribed inflow at the inlet, whose
+// profile values u0(), Tin() are row cj's).  The
 // lattice corners and the cells beyond walls, which several nodes fill,
 // carry zero moments and their populations whole.  Returns false for those.
-template <class C>
-__device__ __forceinline__ bool ghost_moments(const StepParams<C> &p, int ci, int cj, C jx, C jr, C dT, C &gx, C &gr,
-                                              C &gT)
+template <class C, class FU, class FT>
+__device__ __forceinline__ bool ghost_moments(const StepParams<C> &p, int ci, int cj, C jx, C jr, C dT, FU u0, FT Tin,
+                                              C &gx, C &gr, C &gT)
 {
     const bool col_in = ci >= 0 && ci < p.nx, row_in = cj >= 0 && cj < p.nr;
     gx = jx;
@@ -231,9 +243,9 @@ __device__ __forceinline__ bool ghost_moments(const StepParams<C> &p, int ci, in
         return p.bc_top == TOP_OPEN;
     if (row_in && ci == -1) {
         if (p.bc_in == IN_INLET) {
-            gx = p.rho0 * p.u_in[cj];
+            gx = p.rho0 * u0();
             gr = C(0);
-            gT = p.T_in[cj] - p.T0;
+            gT = Tin() - p.T0;
         }
         return true;
     }
@@ -279,6 +291,45 @@ __device__ __forceinline__ double rn_add(double a, double b) { return __dadd_rn(
 __device__ __forceinline__ double rn_sub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double rn_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+template <class C>
+__device__ __forceinline__ C split_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d)
+{
+    if (q == 0)
+        return d;
+    if (q < 9)
+        return rn_fma(C(3) * w9<C>(q), edot<C>(ex9(q), ey9(q), jx, jr), d);
+    return rn_fma(C(0.25), dT, rn_fma(rn_mul(rn_add(p.T0, dT), p.hir0), edot<C>(ex4(q - 9), ey4(q - 9), jx, jr), d));
+}
+
+template <class C>
+__device__ __forceinline__ C split_sub(const StepParams<C> &p, int q, C jx, C jr, C dT, C v)
+{
+    if (q == 0)
+        return v;
+    if (q < 9)
+        return rn_fma(C(-3) * w9<C>(q), edot<C>(ex9(q), ey9(q), jx, jr), v);
+    const C x = rn_mul(rn_add(p.T0, dT), p.hir0);
+    return rn_sub(v, rn_fma(x, edot<C>(ex4(q - 9), ey4(q - 9), jx, jr), rn_mul(C(0.25), dT)));
+}
+
+template <class C>
+__device__ __forceinline__ C edge_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d)
+{
+    if (q < 9)
+        return split_add<C>(p, q, jx, jr, dT, d);
+    const C x = rn_mul(rn_add(p.T0, dT), p.hir0);
+    return rn_add(rn_fma(x, edot<C>(ex4(q - 9), ey4(q - 9), jx, jr), rn_mul(C(0.25), dT)), d);
+}
+
+template <class C>
+__device__ __forceinline__ C edge_sub(const StepParams<C> &p, int q, C jx, C jr, C dT, C v)
+{
+    if (q < 9)
+        return split_sub<C>(p, q, jx, jr, dT, v);
+    const C x = rn_mul(rn_add(p.T0, dT), p.hir0);
+    return rn_sub(v, rn_fma(C(0.25), dT, rn_mul(x, edot<C>(ex4(q - 9), ey4(q - 9), jx, jr))));
+}
 
 template <class C> __device__ __forceinline__ Vec<C, 1> operator+(Vec<C, 1> a, Vec<C, 1> b) { return Vec<C, 1>(rn_add(a.x, b.x)); }
 template <class C> __device__ __forceinline__ Vec<C, 1> operator-(Vec<C, 1> a, Vec<C, 1> b) { return Vec<C, 1>(rn_sub(a.x, b.x)); }
@@ -343,12 +394,11 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x)
     return z ^ (z >> 31);
 }
 
-// prescribed inlet velocity of row j at time index t: profile, plus the
-// noise xi = amp (2U - 1) where the profile is non-zero
+// prescribed inlet velocity of row j at time index t: profile value u, plus
+// the noise xi = amp (2U - 1) where the profile is non-zero
 template <class C>
-__device__ __forceinline__ C inlet_velocity(const StepParams<C> &p, int j, int64_t t)
+__device__ __forceinline__ C noisy_velocity(const StepParams<C> &p, C u, int j, int64_t t)
 {
-    C u = p.u_in[j];
     if (u != C(0) && p.noise_amp != 0.0) {
         const uint64_t c = ((uint64_t)t << 20) + (uint64_t)j;
         const uint64_t h = splitmix64(p.seed ^ splitmix64(c));
@@ -356,6 +406,12 @@ __device__ __forceinline__ C inlet_velocity(const StepParams<C> &p, int j, int64
         u += C(p.noise_amp * (2.0 * U - 1.0));
     }
     return u;
+}
+
+template <class C>
+__device__ __forceinline__ C inlet_velocity(const StepParams<C> &p, int j, int64_t t)
+{
+    return noisy_velocity<C>(p, p.u_in[j], j, t);
 }
 
 // ---- equilibria (deviation form) ---------------------------------------------
@@ -381,14 +437,16 @@ __device__ __forceinline__ C feq_unit(int k, C ux, C ur)
 // The boundary rules of node (i, j) on the lattice edge, given its
 // post-collision deviations fo, go: W(q, ci, cj, v) is called for every
 // ghost cell (ci, cj) of plane q whose value the rules take from this node
-// (v is that value).  t is the time index of the step that will pull these
-// ghosts (inlet noise).  Writers of distinct ghost cells are distinct
-// nodes, except where two rules give the same bounce-back value to the same
-// cell.
-template <class C, class Wr>
+// (v is that value).  U() is row j's prescribed velocity at the step that
+// will pull these ghosts (inlet noise), Tin() its temperature.  PART: 1 the
+// cells beyond the radial edges that depend on no axial rule, 2 the others,
+// 3 both.  Writers of distinct ghost cells are distinct nodes, except where
+// two rules give the same bounce-back value to the same cell.
+template <class C, int PART = 3, class FU, class FT, class Wr>
 __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo)[9], const C (&go)[4], int i, int j,
-                                            int64_t t, Wr W)
+                                            FU U, FT Tin, Wr W)
 {
+    constexpr bool rows = PART & 1, cols = PART & 2;
     const int nx = p.nx, nr = p.nr;
     C drho = C(0), jx = C(0), jr = C(0);
 #pragma unroll
@@ -402,32 +460,34 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
     // zero-gradient copy of this node held at rho0
     auto openc = [&](int k) -> C { return fo[k] - drho * feq_unit<C>(k, ux, ur); };
     // inlet equilibrium at this node's density, this row's prescribed velocity
-    auto inlet_f = [&](int k) -> C { return feq_dev<C>(k, drho, rho, inlet_velocity<C>(p, j, t), C(0)); };
+    auto inlet_f = [&](int k) -> C { return feq_dev<C>(k, drho, rho, U(), C(0)); };
     auto inlet_g0 = [&]() -> C {
-        const C T = p.T_in[j];
-        return C(0.25) * (T - p.T0) + C(0.5) * T * inlet_velocity<C>(p, j, t);
+        const C T = Tin();
+        return rn_fma(C(0.25), T - p.T0, rn_mul(C(0.5) * T, U()));  // (one rounding order in every kernel)
     };
 
     // radial edges (and the corner cells the radial rule reaches first)
     if (j == 0) {
         if (p.bc_bottom == BOTTOM_AXIS) {  // specular mirror
-            W(2, i, -1, fo[4]);
-            W(5, i, -1, fo[8]);
-            W(6, i, -1, fo[7]);
-            W(9 + 1, i, -1, go[3]);
-            if (i == 0) {
+            if (rows) {
+                W(2, i, -1, fo[4]);
+                W(5, i, -1, fo[8]);
+                W(6, i, -1, fo[7]);
+                W(9 + 1, i, -1, go[3]);
+            }
+            if (cols && i == 0) {
                 if (p.bc_in == IN_INLET)
                     W(5, -1, -1, inlet_f(8));
                 else
                     W(6, nx, -1, fo[7]);
             }
-            if (i == nx - 1) {
+            if (cols && i == nx - 1) {
                 if (p.bc_out == OUT_OUTFLOW)
                     W(6, nx, -1, openc(7));
                 else if (p.bc_out == OUT_PERIODIC)
                     W(5, -1, -1, fo[8]);
             }
-        } else {  // half-way bounce-back, thermal anti-bounce-back
+        } else if (rows) {  // half-way bounce-back, thermal anti-bounce-back
             W(2, i, -1, fo[4]);
             W(5, i - 1, -1, fo[7]);
             W(6, i + 1, -1, fo[8]);
@@ -436,22 +496,26 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
     }
     if (j == nr - 1) {
         if (p.bc_top == TOP_WALL) {
-            W(4, i, nr, fo[2]);
-            W(7, i + 1, nr, fo[5]);
-            W(8, i - 1, nr, fo[6]);
-            W(9 + 3, i, nr, -go[1] + C(0.5) * p.dT_top);
+            if (rows) {
+                W(4, i, nr, fo[2]);
+                W(7, i + 1, nr, fo[5]);
+                W(8, i - 1, nr, fo[6]);
+                W(9 + 3, i, nr, -go[1] + C(0.5) * p.dT_top);
+            }
         } else {
-            W(4, i, nr, openc(4));
-            W(7, i, nr, openc(7));
-            W(8, i, nr, openc(8));
-            W(9 + 3, i, nr, go[3]);
-            if (i == 0) {
+            if (rows) {
+                W(4, i, nr, openc(4));
+                W(7, i, nr, openc(7));
+                W(8, i, nr, openc(8));
+                W(9 + 3, i, nr, go[3]);
+            }
+            if (cols && i == 0) {
                 if (p.bc_in == IN_INLET)
                     W(8, -1, nr, inlet_f(8));
                 else
                     W(7, nx, nr, openc(7));
             }
-            if (i == nx - 1) {
+            if (cols && i == nx - 1) {
                 if (p.bc_out == OUT_OUTFLOW)
                     W(7, nx, nr, openc(7));
                 else if (p.bc_out == OUT_PERIODIC)
@@ -460,7 +524,7 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
         }
     }
     // axial edges
-    if (i == 0) {
+    if (cols && i == 0) {
         if (p.bc_in == IN_INLET) {
             W(1, -1, j, inlet_f(1));
             W(5, -1, j, inlet_f(5));
@@ -473,7 +537,7 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
             W(9 + 2, nx, j, go[2]);
         }
     }
-    if (i == nx - 1) {
+    if (cols && i == nx - 1) {
         if (p.bc_out == OUT_OUTFLOW) {
             W(3, nx, j, openc(3));
             W(6, nx, j, openc(6));
@@ -491,6 +555,15 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
             W(9 + 0, -1, j, go[0]);
         }
     }
+}
+
+// t: the time index of the step that will pull these ghosts
+template <class C, class Wr>
+__device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo)[9], const C (&go)[4], int i, int j,
+                                            int64_t t, Wr W)
+{
+    ghost_rules<C>(p, fo, go, i, j, [&]() -> C { return inlet_velocity<C>(p, j, t); },
+                   [&]() -> C { return p.T_in[j]; }, W);
 }
 
 // Two-buffer layout: node (i, j) on the lattice edge, whose post-collision
@@ -516,7 +589,8 @@ __device__ __noinline__ void write_ghosts(const StepParams<C> &p, S *buf, int i,
         ghost_rules<C>(p, fo, go, i, j, t, [&](int q, int ci, int cj, C v) {
             C gx, gr, gT;
             const int64_t oc = cell(p, 0, ci, cj);
-            if (ghost_moments<C>(p, ci, cj, jx, jr, dT, gx, gr, gT)) {
+            if (ghost_moments<C>(p, ci, cj, jx, jr, dT, [&]() -> C { return p.u_in[cj]; },
+                                 [&]() -> C { return p.T_in[cj]; }, gx, gr, gT)) {
                 M.j(oc) = make_float2(gx, gr);
                 M.T(oc) = gT;
                 v -= lin_part<C>(p, q, gx, gr, gT);

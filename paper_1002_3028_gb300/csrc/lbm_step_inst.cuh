@@ -123,6 +123,66 @@ cudaError_t LBM_CAT(occupancy_batch_, LBM_TAG)(int warps_per_cta, int nv, int *c
     return nv == 1 ? occupancy_batch_nv<1>(warps_per_cta, ctas_per_sm) : cudaErrorInvalidValue;
 }
 
+// resident lattices (lbm_resident.cuh): one CTA per tile, all of them resident at once.
+// Two rows a warp in FP32 arithmetic, one in FP64, fill tiles of sixteen rows.
+template <int SHAPE>
+static void res_instance(const void **fn, int *smem)
+{
+    constexpr int NV = LBM_MAX_NV;
+    *fn = reinterpret_cast<const void *>(res_run_kernel<LBM_S, LBM_C, NV, res_rows(SHAPE), res_rpw(SHAPE)>);
+    *smem = res_smem<LBM_S, LBM_C, NV, res_rows(SHAPE)>();
+}
+
+static const void *res_kernel(int shape, int *smem)
+{
+    const void *fn = nullptr;
+    *smem = 0;
+    if (shape == 0)
+        res_instance<0>(&fn, smem);
+#if LBM_MAX_NV > 1
+    if (shape == 1)
+        res_instance<1>(&fn, smem);
+#else
+    if (shape == 2)
+        res_instance<2>(&fn, smem);
+#endif
+    return fn;
+}
+
+cudaError_t LBM_CAT(launch_res_, LBM_TAG)(const StepParams<LBM_C> &p, const ResCtl &ctl, int shape, int warps,
+                                          cudaStream_t s)
+{
+    int smem = 0;
+    const void *fn = res_kernel(shape, &smem);
+    if (!fn)
+        return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ctl.ns * ctl.nb));
+    cfg.blockDim = dim3((unsigned)(32 * warps));
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;  // the CTAs wait on one another
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = ctl.ns * ctl.nb > 1 ? 1 : 0;
+    void *args[2] = {const_cast<StepParams<LBM_C> *>(&p), const_cast<ResCtl *>(&ctl)};
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+cudaError_t LBM_CAT(occupancy_res_, LBM_TAG)(int shape, int warps, int *ctas_per_sm)
+{
+    int smem = 0;
+    const void *fn = res_kernel(shape, &smem);
+    *ctas_per_sm = 0;
+    if (!fn)
+        return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, 32 * warps, (size_t)smem);
+    return e;
+}
+
 cudaError_t LBM_CAT(launch_fields_, LBM_TAG)(const StepParams<LBM_C> &p, void *out, int out_f64, cudaStream_t s)
 {
     const int64_t N = (int64_t)p.nx * p.nr;
