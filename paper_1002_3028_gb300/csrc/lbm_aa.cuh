@@ -524,11 +524,9 @@ __global__ void __launch_bounds__(256) aa_run_kernel(const __grid_constant__ Ste
 template <class S, class C>
 __global__ void aa_fill_ghosts_kernel(const __grid_constant__ StepParams<C> p)
 {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (int64_t)p.nx * p.nr)
-        return;
-    const int i = (int)(n % p.nx), j = (int)(n / p.nx);
-    if (!(i == 0 || i == p.nx - 1 || j == 0 || j == p.nr - 1))
+    int i, j;
+    const int n = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (n >= edge_nodes(p.nx, p.nr) || !edge_node(p.nx, p.nr, n, i, j))
         return;
     S *buf = static_cast<S *>(const_cast<void *>(p.src));
     if (p.phase)
@@ -545,7 +543,7 @@ __host__ __device__ __forceinline__ int64_t aa_post_cell(int phase, int q, int i
     return (int64_t)pq * plane + (int64_t)(cj + 1) * pitch + (ci + PAD_COLS);
 }
 
-// absolute FP64 [q][j][i] <-> the stored deviations (written in representation 0)
+// absolute FP64 [q][j][i] to the stored deviations (written in representation 0)
 template <class S>
 __global__ void aa_state_in_kernel(S *buf, const double *f, const double *g, int nx, int nr, int pitch, int64_t plane,
                                    double rho0, double T0)
@@ -559,24 +557,6 @@ __global__ void aa_state_in_kernel(S *buf, const double *f, const double *g, int
     const int i = (int)(c % nx), j = (int)(c / nx);
     const double v = q < 9 ? f[(int64_t)q * N + c] - w9<double>(q) * rho0 : g[(int64_t)(q - 9) * N + c] - 0.25 * T0;
     buf[aa_post_cell(0, q, i, j, pitch, plane)] = store_as<S, compute_t<S>>(compute_t<S>(v));
-}
-
-template <class S>
-__global__ void aa_state_out_kernel(const S *buf, int phase, double *f, double *g, int nx, int nr, int pitch,
-                                    int64_t plane, double rho0, double T0)
-{
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t N = (int64_t)nx * nr;
-    if (n >= 13 * N)
-        return;
-    const int q = (int)(n / N);
-    const int64_t c = n % N;
-    const int i = (int)(c % nx), j = (int)(c / nx);
-    const double v = (double)load_as<S, compute_t<S>>(buf + aa_post_cell(phase, q, i, j, pitch, plane));
-    if (q < 9)
-        f[(int64_t)q * N + c] = v + w9<double>(q) * rho0;
-    else
-        g[(int64_t)(q - 9) * N + c] = v + 0.25 * T0;
 }
 
 }  // namespace lbm

@@ -1005,10 +1005,10 @@ int finish_diag(const double *v, int have_prev, lbm_diag *out)
     out->mass_axi = v[1];
     out->heat = v[2];
     out->heat_axi = v[3];
-    out->max_speed = v[6];
+    out->max_speed = std::sqrt(v[6]);
     const double nan = std::nan("");
     out->residual_l2 = (have_prev && v[8] > 0.0) ? std::sqrt(v[4] / v[8]) : nan;
-    out->residual_max = (have_prev && v[6] > 0.0) ? v[5] / v[6] : nan;
+    out->residual_max = (have_prev && v[6] > 0.0) ? std::sqrt(v[5]) / std::sqrt(v[6]) : nan;
     out->nonfinite = (int64_t)v[7];
     if (out->nonfinite > 0)
         return fail(LBM_ERR_DIVERGED, "%lld nodes with non-finite or non-positive density or temperature",
@@ -1592,44 +1592,33 @@ int lbm_checkpoint_bytes(const lbm_lattice *h, size_t *bytes)
     return LBM_OK;
 }
 
-// one strided copy per plane between the padded buffer and a dense [q][j][i]
+// the planes between the padded buffer and a dense [q][j][i]
 // array of post-collision values: plane q at its nodes (two buffers), or
 // in the AA pattern the window of the representation's plane that holds
 // population q of every node (lbm::aa_post_cell; restores write
 // representation 0)
 static int copy_planes(lbm_lattice *h, void *dense, bool out, cudaStream_t s)
 {
-    const size_t es = storage_bytes(h->d.storage);
-    const size_t row = (size_t)h->d.nx * es;
-    const size_t pitch = (size_t)h->L.pitch * es;
+    const int64_t es = (int64_t)storage_bytes(h->d.storage);
+    const int nr = h->d.nr;
     char *buf = static_cast<char *>(h->buf(h->cur));
-    const int phase = h->aa && out ? h->phase : 0;
-    for (int q = 0; q < 13; ++q) {
-        const int64_t first = h->aa ? lbm::aa_post_cell(phase, q, 0, 0, h->L.pitch, h->L.plane)
-                                    : (int64_t)q * h->L.plane + h->L.pitch + lbm::PAD_COLS;
-        char *padded = buf + (size_t)first * es;
-        char *flat = static_cast<char *>(dense) + (size_t)q * (size_t)h->d.nr * row;
-        cudaError_t e = out ? cudaMemcpy2DAsync(flat, row, padded, pitch, row, h->d.nr, cudaMemcpyDeviceToDevice, s)
-                            : cudaMemcpy2DAsync(padded, pitch, flat, row, row, h->d.nr, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess)
-            return cuda_fail(e, "checkpoint plane copy");
-    }
+    lbm::PlaneOffsets o = h->aa ? lbm::aa_planes(out ? h->phase : 0, h->L.pitch, h->L.plane)
+                                : lbm::ab_planes(h->L.pitch, h->L.plane);
+    for (int64_t &b : o.off)
+        b *= es;
+    cudaError_t e = lbm::plane_copy(buf, dense, 13, h->d.nx * es, nr, h->L.pitch * es, o, out, s);
     if (is_split(h->d.storage)) {  // then the (j_x, j_r) pairs, then T - T0, without ghosts or padding
         char *mbase = buf + lbm::split_moff(h->L.plane);
-        char *mflat = static_cast<char *>(dense) + (size_t)13 * (size_t)h->d.nr * row;
-        for (int m = 0; m < 2; ++m) {  // m = 0: pairs (8 bytes a node), m = 1: T - T0 (4 bytes)
-            const size_t es_m = m == 0 ? 8 : 4;
-            const size_t mrow = (size_t)h->d.nx * es_m, mpitch = (size_t)h->L.pitch * es_m;
-            char *padded = mbase + (m == 0 ? 0 : (size_t)h->L.plane * 8) +
-                           ((size_t)h->L.pitch + lbm::PAD_COLS) * es_m;
-            char *flat = mflat + (m == 0 ? 0 : (size_t)h->d.nr * (size_t)h->d.nx * 8);
-            cudaError_t e = out ? cudaMemcpy2DAsync(flat, mrow, padded, mpitch, mrow, h->d.nr, cudaMemcpyDeviceToDevice, s)
-                                : cudaMemcpy2DAsync(padded, mpitch, flat, mrow, mrow, h->d.nr, cudaMemcpyDeviceToDevice, s);
-            if (e != cudaSuccess)
-                return cuda_fail(e, "checkpoint moment plane copy");
+        char *mflat = static_cast<char *>(dense) + 13 * (int64_t)nr * h->d.nx * es;
+        for (int m = 0; m < 2 && e == cudaSuccess; ++m) {  // m = 0: pairs (8 bytes a node), m = 1: T - T0 (4 bytes)
+            const int64_t ms = m == 0 ? 8 : 4;
+            o.off[0] = (h->L.pitch + lbm::PAD_COLS) * ms;
+            e = lbm::plane_copy(mbase + (m == 0 ? 0 : h->L.plane * 8),
+                                mflat + (m == 0 ? 0 : (int64_t)nr * h->d.nx * 8), 1, h->d.nx * ms, nr, h->L.pitch * ms,
+                                o, out, s);
         }
     }
-    return LBM_OK;
+    return e == cudaSuccess ? LBM_OK : cuda_fail(e, "checkpoint plane copy");
 }
 
 static int save_impl(lbm_lattice *h, void *dev_out, lbm_stream stream)

@@ -7,6 +7,7 @@
 
 #include "lbm.h"
 #include "lbm_aa_batch.cuh"
+#include "lbm_readout.cuh"
 #include "lbm_resident.cuh"
 
 namespace lbm {

@@ -216,7 +216,7 @@ __device__ __forceinline__ C lin_part(const StepParams<C> &p, int q, C jx, C jr,
 template <class C> __device__ __forceinline__ C split_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d);
 template <class C> __device__ __forceinline__ C split_sub(const StepParams<C> &p, int q, C jx, C jr, C dT, C v);
 // The same with the roundings of write_ghosts: an edge node's populations from what it
-// stored, and what its ghost cells store.
+// stored (a state read out has these too), and what its ghost cells store.
 template <class C> __device__ __forceinline__ C edge_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d);
 template <class C> __device__ __forceinline__ C edge_sub(const StepParams<C> &p, int q, C jx, C jr, C dT, C v);
 
@@ -1650,16 +1650,29 @@ __global__ void advance_kernel(StepParams<C> *lattices, int n, int nsteps)
 }
 
 // ---- ghosts of a stored state (after it is set from outside) ------------------------
+// node n of the lattice's 2 nx + 2 max(nr - 2, 0) edge nodes; false for the repeated ones of
+// one-row and one-column lattices
+__device__ __forceinline__ bool edge_node(int nx, int nr, int n, int &i, int &j)
+{
+    if (n < 2 * nx) {  // bottom row, top row
+        i = n < nx ? n : n - nx;
+        j = n < nx ? 0 : nr - 1;
+        return n < nx || nr > 1;
+    }
+    const int m = n - 2 * nx;  // first and last column between them
+    i = m & 1 ? nx - 1 : 0;
+    j = 1 + (m >> 1);
+    return j < nr - 1 && !((m & 1) && nx == 1);
+}
+__host__ __device__ __forceinline__ int edge_nodes(int nx, int nr) { return 2 * nx + 2 * (nr > 2 ? nr - 2 : 0); }
+
 template <class S, class C>
 __global__ void fill_ghosts_kernel(const __grid_constant__ StepParams<C> p)
 {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (int64_t)p.nx * p.nr)
-        return;
-    const int i = (int)(n % p.nx), j = (int)(n / p.nx);
-    if (!(i == 0 || i == p.nx - 1 || j == 0 || j == p.nr - 1))
-        return;
-    write_ghosts<S, C>(p, static_cast<S *>(p.dst), i, j, p.step);
+    int i, j;
+    const int n = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (n < edge_nodes(p.nx, p.nr) && edge_node(p.nx, p.nr, n, i, j))
+        write_ghosts<S, C>(p, static_cast<S *>(p.dst), i, j, p.step);
 }
 
 // ---- fields at the current time: Eq. 2 moments of the streamed populations ---------------
@@ -1683,40 +1696,62 @@ __global__ void fields_kernel(const __grid_constant__ StepParams<C> p, O *out)
 // Per node, from the populations streamed from the current state (and from
 // the previous state in the other buffer): rho, u, T of Eq. 2.  Sums run in
 // FP64: Σ rho, Σ r rho, Σ T, Σ r T, Σ |u(t) - u(t-1)|^2, Σ |u(t)|^2,
-// max |u(t) - u(t-1)|, max |u(t)|, and the count of nodes whose rho is not
+// max |u(t) - u(t-1)|^2, max |u(t)|^2 (their roots are taken at the end), and the count of nodes whose rho is not
 // finite and positive or whose T is not finite.  Block partials go to
 // `partials` (DIAG_SLOTS doubles per block); diag_final_kernel folds them.
 constexpr int DIAG_SLOTS = 9;
 constexpr int DIAG_THREADS = 256;
 
-__device__ __forceinline__ void diag_combine(double *a, const double *b)
+// GB300 runs two FP64 operations per clock and SM: the sums are FP64, what can be
+// done in integer arithmetic is (conversions from FP32, maxima of values >= 0), and a
+// velocity costs one reciprocal of the density, Newton's from an FP32 start.  The
+// 4096 x 1024 FP32 jet with its previous state: 386 -> 259 us (436 MB, 65 us at the copy
+// rate: still the FP64 unit's time).
+__device__ __forceinline__ double diag_double(double v) { return v; }
+__device__ __forceinline__ double diag_double(float v)
 {
-    for (int k = 0; k < 5; ++k)
-        a[k] += b[k];
-    a[5] = fmax(a[5], b[5]);
-    a[6] = fmax(a[6], b[6]);
-    a[7] += b[7];
-    a[8] += b[8];
+    const unsigned b = __float_as_uint(v), e = b >> 23 & 255u;
+    if (e == 0u || e == 255u)
+        return (double)v;
+    return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3) + (896u << 20)), (int)(b << 29));
+}
+__device__ __forceinline__ double diag_max(double a, double b)  // a, or b if it is a larger number; a >= 0
+{
+    const long long m = __double_as_longlong(b);
+    return m > __double_as_longlong(a) && m <= 0x7ff0000000000000ll ? b : a;
+}
+__device__ __forceinline__ double diag_rcp(double a)
+{
+    double y = (double)(1.f / (float)a);
+    y = fma(y, fma(-a, y, 1.0), y);
+    return fma(y, fma(-a, y, 1.0), y);
 }
 
-// block-wide combine of per-thread slots through shared memory; thread 0 ends with the result
-__device__ __forceinline__ void diag_block_reduce(double (&v)[DIAG_SLOTS])
+__device__ __forceinline__ double diag_combine(int k, double a, double b)
+{
+    return k == 5 || k == 6 ? diag_max(a, b) : a + b;
+}
+
+// block-wide combine of per-thread slots through shared memory; thread k < DIAG_SLOTS ends with slot k
+__device__ __forceinline__ double diag_block_reduce(double (&v)[DIAG_SLOTS])
 {
     __shared__ double sh[DIAG_THREADS / 32][DIAG_SLOTS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int off = 16; off > 0; off >>= 1) {
-        double o[DIAG_SLOTS];
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
         for (int k = 0; k < DIAG_SLOTS; ++k)
-            o[k] = __shfl_down_sync(0xffffffffu, v[k], off);
-        diag_combine(v, o);
-    }
+            v[k] = diag_combine(k, v[k], __shfl_down_sync(0xffffffffu, v[k], off));
     if (lane == 0)
         for (int k = 0; k < DIAG_SLOTS; ++k)
             sh[warp][k] = v[k];
     __syncthreads();
-    if (threadIdx.x == 0)
+    double r = 0.0;
+    if (threadIdx.x < DIAG_SLOTS) {
+        r = sh[0][threadIdx.x];
         for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-            diag_combine(v, sh[w]);
+            r = diag_combine(threadIdx.x, r, sh[w][threadIdx.x]);
+    }
+    return r;
 }
 
 // adds node (i, j) to the per-thread slots
@@ -1724,27 +1759,29 @@ template <class S, class C>
 __device__ __forceinline__ void diag_node(const StepParams<C> &p, int have_prev, int i, int j, double (&v)[DIAG_SLOTS])
 {
     const Mom<Vec<C, 1>> m = node_moments<S, C>(p, i, j, false);
-    const double rho = (double)p.rho0 + (double)m.drho.x;
-    const double T = (double)p.T0 + (double)m.dT.x;
-    const double ux = (double)m.jx.x / rho, ur = (double)m.jr.x / rho;
-    const double r = (double)p.r0 + j + 0.5;
-    if (!(rho > 0.0) || !isfinite(rho) || !isfinite(T) || !isfinite(ux) || !isfinite(ur)) {
+    const double rho = diag_double(p.rho0) + diag_double(m.drho.x);
+    const double T = diag_double(p.T0) + diag_double(m.dT.x);
+    const double jx = diag_double(m.jx.x), jr = diag_double(m.jr.x);
+    if (!(rho > 0.0) || !isfinite(rho) || !isfinite(T) || !isfinite(jx) || !isfinite(jr)) {
         v[7] += 1.0;
         return;
     }
+    const double inv = diag_rcp(rho), ux = jx * inv, ur = jr * inv;
+    const double r = diag_double(p.r0) + j + 0.5;
     v[0] += rho;
     v[1] += r * rho;
     v[2] += T;
     v[3] += r * T;
     const double uu = ux * ux + ur * ur;
     v[8] += uu;
-    v[6] = fmax(v[6], sqrt(uu));
+    v[6] = diag_max(v[6], uu);
     if (have_prev) {
         const Mom<Vec<C, 1>> q = node_moments<S, C>(p, i, j, true);
-        const double rp = (double)p.rho0 + (double)q.drho.x;
-        const double dx = ux - (double)q.jx.x / rp, dr = ur - (double)q.jr.x / rp;
-        v[4] += dx * dx + dr * dr;
-        v[5] = fmax(v[5], sqrt(dx * dx + dr * dr));
+        const double ip = diag_rcp(diag_double(p.rho0) + diag_double(q.drho.x));
+        const double dx = ux - diag_double(q.jx.x) * ip, dr = ur - diag_double(q.jr.x) * ip;
+        const double dd = dx * dx + dr * dr;
+        v[4] += dd;
+        v[5] = diag_max(v[5], dd);
     }
 }
 
@@ -1753,13 +1790,14 @@ __global__ void __launch_bounds__(DIAG_THREADS) diag_kernel(const __grid_constan
                                                             double *partials)
 {
     double v[DIAG_SLOTS] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    const int64_t N = (int64_t)p.nx * p.nr;
-    for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x)
-        diag_node<S, C>(p, have_prev, (int)(n % p.nx), (int)(n / p.nx), v);
-    diag_block_reduce(v);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < DIAG_SLOTS; ++k)
-            partials[(int64_t)blockIdx.x * DIAG_SLOTS + k] = v[k];
+    const unsigned N = (unsigned)p.nx * (unsigned)p.nr, step = gridDim.x * blockDim.x;
+    for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += step) {
+        const unsigned j = n / (unsigned)p.nx;
+        diag_node<S, C>(p, have_prev, (int)(n - j * (unsigned)p.nx), (int)j, v);
+    }
+    const double r = diag_block_reduce(v);
+    if (threadIdx.x < DIAG_SLOTS)
+        partials[(int64_t)blockIdx.x * DIAG_SLOTS + threadIdx.x] = r;
 }
 
 // one block folds nblocks partials into out[0 .. DIAG_SLOTS-1]
@@ -1767,14 +1805,15 @@ static __global__ void __launch_bounds__(DIAG_THREADS) diag_final_kernel(const d
 {
     double v[DIAG_SLOTS] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-        diag_combine(v, partials + (int64_t)b * DIAG_SLOTS);
-    diag_block_reduce(v);
-    if (threadIdx.x == 0)
+#pragma unroll
         for (int k = 0; k < DIAG_SLOTS; ++k)
-            out[k] = v[k];
+            v[k] = diag_combine(k, v[k], partials[(int64_t)b * DIAG_SLOTS + k]);
+    const double r = diag_block_reduce(v);
+    if (threadIdx.x < DIAG_SLOTS)
+        out[threadIdx.x] = r;
 }
 
-// ---- state conversion: absolute FP64 [q][j][i] <-> stored deviations -----------------
+// ---- state conversion: absolute FP64 [q][j][i] to stored deviations (out: lbm_readout.cuh) --
 template <class S>
 using compute_t = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
 
@@ -1795,25 +1834,6 @@ __global__ void state_in_kernel(S *buf, const double *f, const double *g, int nx
     else
         v = g[(int64_t)(q - 9) * N + c] - 0.25 * T0;
     buf[(int64_t)q * plane + (int64_t)(j + 1) * pitch + (i + PAD_COLS)] = store_as<S, compute_t<S>>(compute_t<S>(v));
-}
-
-template <class S>
-__global__ void state_out_kernel(const S *buf, double *f, double *g, int nx, int nr, int pitch, int64_t plane,
-                                 double rho0, double T0)
-{
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t N = (int64_t)nx * nr;
-    if (n >= 13 * N)
-        return;
-    const int q = (int)(n / N);
-    const int64_t c = n % N;
-    const int i = (int)(c % nx), j = (int)(c / nx);
-    const double v =
-        (double)load_as<S, compute_t<S>>(buf + (int64_t)q * plane + (int64_t)(j + 1) * pitch + (i + PAD_COLS));
-    if (q < 9)
-        f[(int64_t)q * N + c] = v + w9<double>(q) * rho0;
-    else
-        g[(int64_t)(q - 9) * N + c] = v + 0.25 * T0;
 }
 
 // ---- moment-split storage: state conversion, one node per thread ----------------------
@@ -1854,29 +1874,6 @@ __global__ void split_state_in_kernel(S *buf, const double *f, const double *g, 
     M.T(o) = mT;
     for (int q = 0; q < 13; ++q)
         buf[(int64_t)q * plane + o] = store_as<S, float>(float(dev[q]) - lin_part<float>(lp, q, mx, mr, mT));
-}
-
-template <class S>
-__global__ void split_state_out_kernel(const S *buf, double *f, double *g, int nx, int nr, int pitch, int64_t plane,
-                                       double rho0, double T0)
-{
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t N = (int64_t)nx * nr;
-    if (n >= N)
-        return;
-    const int i = (int)(n % nx), j = (int)(n / nx);
-    const StepParams<float> lp = lin_params(rho0, T0);
-    const int64_t o = (int64_t)(j + 1) * pitch + (i + PAD_COLS);
-    const float *M = split_m(buf, plane);
-    const float2 jj = reinterpret_cast<const float2 *>(M)[o];
-    const float mx = jj.x, mr = jj.y, mT = M[2 * plane + o];
-    for (int q = 0; q < 13; ++q) {
-        const double v = double(lin_part<float>(lp, q, mx, mr, mT) + load_as<S, float>(buf + (int64_t)q * plane + o));
-        if (q < 9)
-            f[(int64_t)q * N + n] = v + w9<double>(q) * rho0;
-        else
-            g[(int64_t)(q - 9) * N + n] = v + 0.25 * T0;
-    }
 }
 
 }  // namespace lbm

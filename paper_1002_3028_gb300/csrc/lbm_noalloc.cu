@@ -69,10 +69,9 @@ __global__ void __launch_bounds__(DIAG_THREADS) diag_rows_kernel(const __grid_co
     const int j = blockIdx.x;
     for (int i = threadIdx.x; i < p.nx; i += blockDim.x)
         diag_node<S, C>(p, have_prev, i, j, v);
-    diag_block_reduce(v);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < DIAG_SLOTS; ++k)
-            partials[(int64_t)j * DIAG_SLOTS + k] = v[k];
+    const double r = diag_block_reduce(v);
+    if (threadIdx.x < DIAG_SLOTS)
+        partials[(int64_t)j * DIAG_SLOTS + threadIdx.x] = r;
 }
 
 template <class S, class C>

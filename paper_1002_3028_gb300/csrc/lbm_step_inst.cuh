@@ -197,9 +197,8 @@ cudaError_t LBM_CAT(launch_fields_, LBM_TAG)(const StepParams<LBM_C> &p, void *o
 
 cudaError_t LBM_CAT(launch_fill_, LBM_TAG)(const StepParams<LBM_C> &p, cudaStream_t s)
 {
-    const int64_t N = (int64_t)p.nx * p.nr;
-    const int threads = 256;
-    fill_ghosts_kernel<LBM_S, LBM_C><<<(unsigned)((N + threads - 1) / threads), threads, 0, s>>>(p);
+    const int threads = 64;  // an edge node per thread, spread over the SMs
+    fill_ghosts_kernel<LBM_S, LBM_C><<<(edge_nodes(p.nx, p.nr) + threads - 1) / threads, threads, 0, s>>>(p);
     return cudaGetLastError();
 }
 
@@ -234,15 +233,17 @@ cudaError_t LBM_CAT(launch_state_in_, LBM_TAG)(void *buf, const double *f, const
 cudaError_t LBM_CAT(launch_state_out_, LBM_TAG)(const void *buf, double *f, double *g, int nx, int nr, int pitch,
                                                 int64_t plane, double rho0, double T0, cudaStream_t s)
 {
-    const int threads = 256;
 #ifdef LBM_SPLIT
-    const int64_t n = (int64_t)nx * nr;
-    split_state_out_kernel<LBM_S><<<(unsigned)((n + threads - 1) / threads), threads, 0, s>>>(
-        static_cast<const LBM_S *>(buf), f, g, nx, nr, pitch, plane, rho0, T0);
+    // up to eight rows a thread (its constants once), as long as some thousand CTAs remain
+    const int across = (nx + 255) / 256;
+    const int64_t rows = (int64_t)across * nr / 1216;
+    const int per = (int)(rows < 1 ? 1 : (rows > 8 ? 8 : rows)), up = (nr + per - 1) / per;
+    const dim3 grid((unsigned)across, (unsigned)(up < 65535 ? up : 65535));
+    split_state_out_kernel<LBM_S><<<grid, 256, 0, s>>>(static_cast<const LBM_S *>(buf), f, g, nx, nr, pitch, plane,
+                                                       rho0, T0);
 #else
-    const int64_t n = 13 * (int64_t)nx * nr;
-    state_out_kernel<LBM_S><<<(unsigned)((n + threads - 1) / threads), threads, 0, s>>>(
-        static_cast<const LBM_S *>(buf), f, g, nx, nr, pitch, plane, rho0, T0);
+    state_out_kernel<LBM_S><<<read_blocks(13 * nr, nx), 256, 0, s>>>(static_cast<const LBM_S *>(buf), f, g, nx, nr,
+                                                                     pitch, ab_planes(pitch, plane), rho0, T0);
 #endif
     return cudaGetLastError();
 }
@@ -298,9 +299,8 @@ cudaError_t LBM_CAT(occupancy_aa_batch_, LBM_TAG)(int warps_per_cta, int *ctas_p
 
 cudaError_t LBM_CAT(launch_aa_fill_, LBM_TAG)(const StepParams<LBM_C> &p, cudaStream_t s)
 {
-    const int64_t N = (int64_t)p.nx * p.nr;
-    const int threads = 256;
-    aa_fill_ghosts_kernel<LBM_S, LBM_C><<<(unsigned)((N + threads - 1) / threads), threads, 0, s>>>(p);
+    const int threads = 64;
+    aa_fill_ghosts_kernel<LBM_S, LBM_C><<<(edge_nodes(p.nx, p.nr) + threads - 1) / threads, threads, 0, s>>>(p);
     return cudaGetLastError();
 }
 
@@ -317,10 +317,8 @@ cudaError_t LBM_CAT(launch_aa_state_in_, LBM_TAG)(void *buf, const double *f, co
 cudaError_t LBM_CAT(launch_aa_state_out_, LBM_TAG)(const void *buf, int phase, double *f, double *g, int nx, int nr,
                                                    int pitch, int64_t plane, double rho0, double T0, cudaStream_t s)
 {
-    const int64_t n = 13 * (int64_t)nx * nr;
-    const int threads = 256;
-    aa_state_out_kernel<LBM_S><<<(unsigned)((n + threads - 1) / threads), threads, 0, s>>>(
-        static_cast<const LBM_S *>(buf), phase, f, g, nx, nr, pitch, plane, rho0, T0);
+    state_out_kernel<LBM_S><<<read_blocks(13 * nr, nx), 256, 0, s>>>(static_cast<const LBM_S *>(buf), f, g, nx, nr,
+                                                                     pitch, aa_planes(phase, pitch, plane), rho0, T0);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,76 @@
+"""Reading a state out: FP64 populations formed in integer arithmetic (csrc/lbm_readout.cuh) have
+the bits of the FP64 sum, and checkpoints copied in wide or narrow words hold the same values."""
+import numpy as np
+import pytest
+
+from paper_1002_3028_gb300 import inputs as I
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+W9 = [4 / 9] + [1 / 9] * 4 + [1 / 36] * 4
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1002_3028_gb300 import lbm as L
+
+    L.lib()
+    return L
+
+
+def deviations(shape, seed):
+    """Deviations of every size and sign: around the constants' binade edges, up to several times
+    the constants, down to far below their last place, and exact zeros."""
+    rng = np.random.default_rng(seed)
+    mag = np.exp(rng.uniform(np.log(1e-25), np.log(8.0), shape))
+    v = mag * rng.choice([-1.0, 1.0], shape)
+    v[rng.random(shape) < 0.05] = 0.0
+    near = rng.random(shape) < 0.2
+    edges = np.array([0.5, 0.25, 0.125, 0.0625, 0.03125, 0.015625])
+    c = np.array(W9 + [0.25] * 4).reshape(13, 1, 1)
+    v = np.where(near, rng.choice(edges, shape) - c + 1e-7 * rng.standard_normal(shape), v)
+    return v
+
+
+@pytest.mark.parametrize("rho0,T0", [(1.0, 1.0), (1.0, 0.7), (1.3, 1.0)])
+@pytest.mark.parametrize("storage,pattern", [("f32", "ab"), ("f16", "ab"), ("bf16", "ab"), ("f32", "aa"), ("f16s", "ab")])
+@pytest.mark.parametrize("size", [(300, 41), (33, 3)], ids=lambda s: f"{s[0]}x{s[1]}")
+def test_fp64_populations_are_the_fp64_sums(lbm, size, storage, pattern, rho0, T0):
+    nx, nr = size
+    cfg = I.LatticeConfig(nx=nx, nr=nr, rho0=rho0, T0=T0)
+    lat = lbm.Lattice(cfg, storage, device="cuda:0", pattern=pattern)
+    c = np.array([w * rho0 for w in W9] + [0.25 * T0] * 4).reshape(13, 1, 1)
+    a = c + deviations((13, nr, nx), 5)
+    lat.set_state(a[:9], a[9:])
+    f, g = lat.get_state()
+    got = torch.cat([f, g]).cpu().numpy()
+    planes = lat.save()[0]
+    if storage == "f16s":  # the stored values are not deviations from rest: one FP32 rounding from them
+        assert np.all(np.abs(got - a) <= 2e-3 * np.abs(a - c) + 2e-2)
+        assert np.array_equal(got, (got - c).astype(np.float32).astype(np.float64) + c) or rho0 != 1.0
+        return
+    want = planes.cpu().double().numpy() + c
+    if rho0 == 1.0:
+        assert np.array_equal(got, want)
+    else:  # the product w rho0 rounds, or is fused into the sum
+        assert np.allclose(got, want, rtol=0, atol=4e-16 * 8)
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32", "f16", "f16s"])
+@pytest.mark.parametrize("nx", [1, 7, 64, 130, 301, 520])
+@pytest.mark.parametrize("pattern,steps", [("ab", 3), ("aa", 2), ("aa", 3)])
+def test_checkpoints_of_every_row_alignment(lbm, nx, storage, pattern, steps):
+    if storage == "f16s" and pattern == "aa":
+        pytest.skip("moment-split storage has no AA pattern")
+    w = I.jet_workload(nx=nx, nr=11)
+    a, b = (lbm.Lattice.from_workload(w, storage, device="cuda:0", pattern=pattern) for _ in range(2))
+    a.step(steps)
+    planes, step = a.save()
+    b.restore(planes, step)
+    assert torch.equal(a.fields(), b.fields())
+    a.step(2)
+    b.step(2)
+    assert torch.equal(a.save()[0], b.save()[0])
