@@ -11,7 +11,8 @@
 // within its binade, so while the sum stays in the constant's binade its bits
 // are the constant's plus the deviation rounded to those units.  Sums that
 // leave it (deviations of the order of the constant, in the core of a hot
-// jet) take the FP64 operations.  Same bits either way.
+// jet) take the FP64 operations.  Same bits either way.  4096 x 1024: FP32
+// 241 -> 123 us, FP16 moment-split 300 -> 124 (98 and 89 us at the copy rate).
 #pragma once
 
 #include "lbm_aa.cuh"
@@ -158,7 +159,7 @@ inline unsigned read_blocks(int rows, int nx)
 // ---- checkpoints ---------------------------------------------------------------------
 // Rows of `planes` planes between the padded buffer and a dense [plane][row][n]
 // array, in words of type U.  One launch instead of a strided copy per plane
-// (4096 x 1024 FP32: 13 copies took 290 us for 436 MB).
+// (4096 x 1024 FP32, 436 MB: 13 copies some 290 us, this 60).
 template <class U, bool OUT>
 __global__ void __launch_bounds__(256) plane_copy_kernel(U *padded, U *dense, int planes, int n, int nr, int pitch,
                                                          const __grid_constant__ PlaneOffsets offs)
