@@ -461,10 +461,11 @@ int plan_launch(lbm_lattice *h)
 // Lattices that fit the chip run their steps there (lbm_resident.cuh): strips of 64 columns
 // (FP64 32), cut into tiles of one CTA each, every CTA resident.  Of the tile shapes, in FP32
 // arithmetic: eight rows, one a warp, while one tile a SM is enough (us per step: 200 x 96
-// FP32 3.8 with tiles of 8 rows, 4.2 of 6, 4.5 of 4, 6.1 of 16 rows with two rows a warp);
+// FP32 3.4 with tiles of 8 rows; 0.4 more in tiles of 6, 0.7 of 4, 2.3 of 16 rows with two
+// rows a warp);
 // then the same with two CTAs a SM, whose registers leave room for six warps each
-// (640 x 160 FP16 moment-split 6.4 in tiles of 5 and 6 rows, 7.4 of 14 with two rows a warp);
-// then sixteen rows, two a warp, two CTAs a SM (1024 x 256 FP32 7.4).  FP64 is bound by its
+// (640 x 160 FP16 moment-split 4.5 in tiles of 5 and 6 rows, 1.0 more of 14 with two rows a
+// warp); then sixteen rows, two a warp, two CTAs a SM (1024 x 256 FP32 6.0).  FP64 is bound by its
 // arithmetic: the tiles that spread it over the SMs best.  The step kernel takes 8.8, 15.8
 // and 12.4 us on the three lattices and keeps those that do not fit, those with periodic
 // ends or in the AA layout, and those whose launch shape the caller has set.

@@ -438,15 +438,15 @@ __device__ __forceinline__ C feq_unit(int k, C ux, C ur)
 // post-collision deviations fo, go: W(q, ci, cj, v) is called for every
 // ghost cell (ci, cj) of plane q whose value the rules take from this node
 // (v is that value).  U() is row j's prescribed velocity at the step that
-// will pull these ghosts (inlet noise), Tin() its temperature.  PART: 1 the
-// cells beyond the radial edges that depend on no axial rule, 2 the others,
-// 3 both.  Writers of distinct ghost cells are distinct nodes, except where
+// will pull these ghosts (inlet noise), Tin() its temperature.  SIDES: which
+// edges' rules are applied (1 first column, 2 last column, with the corner
+// cells that a radial rule reaches first; 4 bottom row, 8 top row).  Writers of distinct ghost cells are distinct nodes, except where
 // two rules give the same bounce-back value to the same cell.
-template <class C, int PART = 3, class FU, class FT, class Wr>
+template <class C, int SIDES = 15, class FU, class FT, class Wr>
 __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo)[9], const C (&go)[4], int i, int j,
                                             FU U, FT Tin, Wr W)
 {
-    constexpr bool rows = PART & 1, cols = PART & 2;
+    constexpr bool first = SIDES & 1, last = SIDES & 2, bottom = SIDES & 4, top = SIDES & 8;
     const int nx = p.nx, nr = p.nr;
     C drho = C(0), jx = C(0), jr = C(0);
 #pragma unroll
@@ -469,25 +469,25 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
     // radial edges (and the corner cells the radial rule reaches first)
     if (j == 0) {
         if (p.bc_bottom == BOTTOM_AXIS) {  // specular mirror
-            if (rows) {
+            if (bottom) {
                 W(2, i, -1, fo[4]);
                 W(5, i, -1, fo[8]);
                 W(6, i, -1, fo[7]);
                 W(9 + 1, i, -1, go[3]);
             }
-            if (cols && i == 0) {
+            if (first && i == 0) {
                 if (p.bc_in == IN_INLET)
                     W(5, -1, -1, inlet_f(8));
                 else
                     W(6, nx, -1, fo[7]);
             }
-            if (cols && i == nx - 1) {
+            if (last && i == nx - 1) {
                 if (p.bc_out == OUT_OUTFLOW)
                     W(6, nx, -1, openc(7));
                 else if (p.bc_out == OUT_PERIODIC)
                     W(5, -1, -1, fo[8]);
             }
-        } else if (rows) {  // half-way bounce-back, thermal anti-bounce-back
+        } else if (bottom) {  // half-way bounce-back, thermal anti-bounce-back
             W(2, i, -1, fo[4]);
             W(5, i - 1, -1, fo[7]);
             W(6, i + 1, -1, fo[8]);
@@ -496,26 +496,26 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
     }
     if (j == nr - 1) {
         if (p.bc_top == TOP_WALL) {
-            if (rows) {
+            if (top) {
                 W(4, i, nr, fo[2]);
                 W(7, i + 1, nr, fo[5]);
                 W(8, i - 1, nr, fo[6]);
                 W(9 + 3, i, nr, -go[1] + C(0.5) * p.dT_top);
             }
         } else {
-            if (rows) {
+            if (top) {
                 W(4, i, nr, openc(4));
                 W(7, i, nr, openc(7));
                 W(8, i, nr, openc(8));
                 W(9 + 3, i, nr, go[3]);
             }
-            if (cols && i == 0) {
+            if (first && i == 0) {
                 if (p.bc_in == IN_INLET)
                     W(8, -1, nr, inlet_f(8));
                 else
                     W(7, nx, nr, openc(7));
             }
-            if (cols && i == nx - 1) {
+            if (last && i == nx - 1) {
                 if (p.bc_out == OUT_OUTFLOW)
                     W(7, nx, nr, openc(7));
                 else if (p.bc_out == OUT_PERIODIC)
@@ -524,7 +524,7 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
         }
     }
     // axial edges
-    if (cols && i == 0) {
+    if (first && i == 0) {
         if (p.bc_in == IN_INLET) {
             W(1, -1, j, inlet_f(1));
             W(5, -1, j, inlet_f(5));
@@ -537,7 +537,7 @@ __device__ __forceinline__ void ghost_rules(const StepParams<C> &p, const C (&fo
             W(9 + 2, nx, j, go[2]);
         }
     }
-    if (cols && i == nx - 1) {
+    if (last && i == nx - 1) {
         if (p.bc_out == OUT_OUTFLOW) {
             W(3, nx, j, openc(3));
             W(6, nx, j, openc(6));

@@ -20,20 +20,20 @@
 // release and the neighbours' acquire.  Here a step is two barriers, one
 // collision's latency per row a warp holds, and the exchange of the ring.
 // us per step, the step kernel against this one (200 steps a launch):
-// 64 x 32 FP32 6.7 -> 3.6, 200 x 96 FP32 8.8 -> 3.8 and FP64 19.5 -> 16.9,
-// 512 x 128 FP32 10.3 -> 3.9, 640 x 160 FP16 moment-split 15.8 -> 6.4,
-// 1024 x 256 FP32 12.4 -> 7.4 and FP16 moment-split 17.5 -> 10.4.  With the
-// exchange's waits taken out the last three would take 4.6 us in FP32: the
-// rest is the way of a value through L2 and the slowest tile of each
-// neighbourhood.
+// 64 x 32 FP32 6.7 -> 3.3, 200 x 96 FP32 8.8 -> 3.4 and FP64 19.5 -> 16.2,
+// 640 x 160 FP16 moment-split 15.8 -> 4.5, 777 x 301 17.9 -> 7.6,
+// 1024 x 256 FP32 12.4 -> 6.0.  With the exchange's waits taken out the last
+// takes 4.6: the rest is the way of a value through L2 and the slowest tile
+// of each neighbourhood, one at a lattice edge, whose ghosts come after its
+// collisions.
 //
 // Exchange.  A tile sends the values that the rings of the eight tiles
 // around it hold straight to their inboxes in device memory, each in one
 // 8-byte word with the number of its step: a reader polls the values
 // themselves, so a step costs one store and one load across L2 and no fence,
 // flag or extra round trip.  (With the ring kept in the lattice's buffers
-// and flags released after the stores, 1024 x 256 FP32 took 12.4 us a step,
-// of which the fence, the flag and the loads after it were more than 3.)  An
+// and flags released after the stores, 1024 x 256 FP32 took 5 us a step
+// longer.)  An
 // inbox has two halves, for even and odd steps: a tile sends step k + 2 only
 // after it has read every neighbour's step k + 1, which was sent after the
 // neighbour had read step k.
@@ -82,6 +82,7 @@ __host__ __device__ constexpr int res_rows(int shape) { return shape == 0 ? 8 : 
 __host__ __device__ constexpr int res_rpw(int shape) { return shape == 1 ? 2 : 1; }
 
 constexpr int RES_CORNERS = 32;     // corner entries of an inbox (res_corner; two unused)
+constexpr int RES_EDGES = 6;        // tasks of filling ghosts: left, right, bottom and top in halves of 32 columns
 constexpr int RES_SEND_MAX = 96;    // corner entries a tile sends
 
 // a tile's shared memory: 13 planes of populations with a ring of two cells,
@@ -115,6 +116,8 @@ struct ResMem {
     // corner entries to send: (offset in pop, who sends it) and the destination word; their number
     __device__ __forceinline__ int2 *send() const { return reinterpret_cast<int2 *>(raw + VALUES + TAB); }
     __device__ __forceinline__ int &nsend() const { return *reinterpret_cast<int *>(send() + RES_SEND_MAX); }
+    // entries of the inbox that a warp has taken charge of in this step
+    __device__ __forceinline__ int &taken() const { return (&nsend())[1]; }
     // where each entry received goes (an offset from the first value), or RES_NONE
     __device__ __forceinline__ unsigned short *recv() const
     {
@@ -223,8 +226,8 @@ __device__ __forceinline__ void res_writer(const StepParams<C> &p, int q, int i,
 }
 
 // Lists where the entries the tile receives go, and the corner entries it
-// sends.  An entry sent is tagged with its sender: the warp that holds the node's row, or 64 + the
-// edge (0 left, 1 right, 2 bottom, 3 top) whose ghost it is.
+// sends.  An entry sent is tagged with its sender: the warp that holds the
+// node's row, or 64 + the edge task (RES_EDGES) whose ghost it is.
 template <class C, int NV, int TH, int RPW>
 __device__ __noinline__ void res_lists(const StepParams<C> &p, const int ns, const int nb, const ResTile a)
 {
@@ -276,9 +279,9 @@ __device__ __noinline__ void res_lists(const StepParams<C> &p, const int ns, con
             continue;
         int who = (j - a.j0) / RPW;
         if (i < 0 || i >= p.nx)
-            who = 64 + (wi == 0 ? 0 : 1);
+            who = 64 + (i < 0 ? 0 : 1);
         else if (j < 0 || j >= p.nr)
-            who = 64 + (wj == 0 ? 2 : 3);
+            who = 64 + (j < 0 ? 2 : 4) + (wi - a.x0 >= 32);
         const int m = atomicAdd(&t.nsend(), 1);
         if (m < RES_SEND_MAX)
             t.send()[m] = make_int2((x.q * Mem::PL + (j - a.j0) * Mem::PW + (i - a.x0) + 1024) | who << 20,
@@ -298,10 +301,12 @@ __device__ __forceinline__ bool res_poll_again(const StepParams<C> &p, int spin_
     return true;
 }
 
-// Receives the ring of state number seq: every thread polls its share of the
-// inbox, a few entries at a time, and puts each value where the tile's table
-// says.  (One unrolled loop per kind of ring row and column instead of the
-// table cost the kernel 80 registers.)
+// Receives the ring of state number seq: warps take pieces of the inbox until
+// none is left (one that fills ghosts comes late and finds less to do), and
+// every thread polls its entries of a piece and puts each value where the
+// tile's table says.  (One unrolled loop per kind of ring row and column
+// instead of the table cost the kernel 80 registers; pieces of 8 entries a
+// thread took 7.8 us a step on the 1024 x 256 FP32 jet, of 4 7.4, of 2 7.6.)
 template <class C, int NV, int TH>
 __device__ __noinline__ bool res_receive(const StepParams<C> &p, const int spin_limit, const unsigned long long *box,
                                          unsigned seq)
@@ -309,14 +314,21 @@ __device__ __noinline__ bool res_receive(const StepParams<C> &p, const int spin_
     using Mem = ResMem<C, NV, TH>;
     constexpr int B = 4;
     const Mem t;
+    const int lane = threadIdx.x & 31;
     C *cells = reinterpret_cast<C *>(t.raw);
-#pragma unroll 1
-    for (int e0 = threadIdx.x; e0 - (int)(threadIdx.x & 31u) < Mem::ENTRIES; e0 += B * blockDim.x) {
+    for (;;) {
+        int e0 = 0;
+        if (lane == 0)
+            e0 = atomicAdd(&t.taken(), 32 * B);
+        e0 = __shfl_sync(0xffffffffu, e0, 0);
+        if (e0 >= Mem::ENTRIES)
+            return true;
+        e0 += lane;
         int off[B];
         C v[B];
 #pragma unroll
         for (int n = 0; n < B; ++n) {
-            const int e = e0 + n * blockDim.x;
+            const int e = e0 + 32 * n;
             off[n] = e < Mem::ENTRIES ? t.recv()[e] : RES_NONE;
         }
         // (only what has not come yet is read again: polls compete with the values on their way)
@@ -331,7 +343,7 @@ __device__ __noinline__ bool res_receive(const StepParams<C> &p, const int spin_
             for (int n = 0; n < B; ++n) {
                 if (!got[n]) {
                     got[n] = true;
-                    v[n] = box_get<C>(box + (e0 + n * blockDim.x) * Mem::WPV, seq, got[n]);
+                    v[n] = box_get<C>(box + (e0 + 32 * n) * Mem::WPV, seq, got[n]);
                 }
             }
 #pragma unroll
@@ -347,7 +359,6 @@ __device__ __noinline__ bool res_receive(const StepParams<C> &p, const int spin_
             if (off[n] != RES_NONE)
                 cells[off[n]] = v[n];
     }
-    return true;
 }
 
 // sends the corner entries tagged `who`
@@ -473,10 +484,15 @@ __host__ __device__ constexpr int res_smem()
     return ResMem<C, NV, TH>::BYTES + (IsSplit<S>::value ? 4 * (2 * TH + 64 * NV) * (int)sizeof(C) : 0);
 }
 
-// Ghost cells of lattice-edge node (r, c) of the tile, from its populations
-// in shared memory: into the tile's ring and, with dst, into that state; the
-// row's inlet velocity with noise, without, and temperature.  PART: of ghost_rules.
-template <class S, class C, int NV, int TH, int PART>
+// Ghost cells of lattice-edge node (r, c) of the tile beyond one edge (SIDE: 0
+// first column, 1 last column, 2 bottom row, 3 top row), from its populations
+// in shared memory: into the tile's ring and, with OUT, into the state dst;
+// the row's inlet velocity with noise, without, and temperature.  These are
+// the longest chain of a step of a tile at a lattice edge, for which its
+// neighbours wait: one edge and no stored state at a time leaves the least of
+// it (filling all of a node's ghosts in one call cost 777 x 301 FP16
+// moment-split 1.6 of 10.2 us a step, 640 x 160 2.1 of 6.4).
+template <class S, class C, int NV, int TH, int SIDE, bool OUT>
 __device__ __noinline__ void res_ghosts(const StepParams<C> &p, S *dst, const int x0, const int j0, int r, int c, C uin,
                                         C u0, C Tin)
 {
@@ -490,43 +506,78 @@ __device__ __noinline__ void res_ghosts(const StepParams<C> &p, S *dst, const in
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         go[k] = own[(9 + k) * Mem::PL];
-    C jx = C(0), jr = C(0), dT = C(0);
+    // moment-split storage: the moments the ghost cells carry (ghost_moments), if any
+    C gx = C(0), gr = C(0), gT = C(0);
+    bool carried = false;
     if constexpr (IsSplit<S>::value) {
         const C *eg = res_edge_g<C, NV, TH>(t, p, x0 + c, j0 + r, r, c);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             go[k] = eg[k];
-        jx = t.M(0, r, c);
-        jr = t.M(1, r, c);
-        dT = t.M(2, r, c);
+        if (SIDE == 0) {
+            gx = p.rho0 * u0;
+            gT = Tin - p.T0;
+            carried = true;
+        } else {
+            gx = t.M(0, r, c);
+            gr = SIDE == 2 ? -t.M(1, r, c) : t.M(1, r, c);
+            gT = t.M(2, r, c);
+            carried = SIDE == 1 ? p.bc_out != OUT_WALL
+                                : (SIDE == 2 ? p.bc_bottom == BOTTOM_AXIS : p.bc_top == TOP_OPEN);
+        }
     }
     const int pl = (int)p.plane;
     auto W = [&](int q, int ci, int cj, C v) {
         S s;
         const int o = (cj + 1) * p.pitch + ci + PAD_COLS;
-        if constexpr (IsSplit<S>::value) {
-            C gx, gr, gT;
-            if (ghost_moments<C>(p, ci, cj, jx, jr, dT, [&]() -> C { return u0; }, [&]() -> C { return Tin; }, gx, gr,
-                                 gT)) {
-                if (dst) {
+        // the lattice's corner cells and those beyond walls: no moments, the population whole
+        if (IsSplit<S>::value && carried && (SIDE > 1 || (cj >= 0 && cj < p.nr))) {
+            if constexpr (IsSplit<S>::value) {
+                if constexpr (OUT) {
                     const MomRef M{split_m(dst, p.plane), p.plane};
                     M.j(o) = make_float2(gx, gr);
                     M.T(o) = gT;
                 }
                 s = store_as<S, C>(edge_sub<C>(p, q, gx, gr, gT, v));
                 v = split_add<C>(p, q, gx, gr, gT, load_as_shared<S, C>(&s));
-            } else {  // zero moments: the population whole
-                s = store_as<S, C>(v);
-                v = load_as_shared<S, C>(&s);
             }
         } else {
-            v = res_round<S, C>(p, q, v, C(0), C(0), C(0), s);
+            s = store_as<S, C>(v);
+            v = load_as_shared<S, C>(&s);
         }
         t.P(q, cj - j0, ci - x0) = v;
-        if (dst)
+        if constexpr (OUT)
             dst[o + q * pl] = s;
     };
-    ghost_rules<C, PART>(p, fo, go, x0 + c, j0 + r, [&]() -> C { return uin; }, [&]() -> C { return Tin; }, W);
+    ghost_rules<C, 1 << SIDE>(p, fo, go, x0 + c, j0 + r, [&]() -> C { return uin; }, [&]() -> C { return Tin; }, W);
+}
+
+__device__ __forceinline__ void named_barrier(int id, bool wait)
+{
+    if (wait)
+        asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"((int)blockDim.x) : "memory");
+    else
+        asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"((int)blockDim.x) : "memory");
+}
+
+// edge task n of a tile: one lane per node
+template <class S, class C, int NV, int TH, bool OUT>
+__device__ __forceinline__ void res_edge_task(const StepParams<C> &p, S *dst, const ResTile &a, int n, C uin, C u0,
+                                              C Tin)
+{
+    const int lane = threadIdx.x & 31, c = lane + 32 * (n & 1);
+    if (n == 0) {
+        if (lane < a.h)
+            res_ghosts<S, C, NV, TH, 0, OUT>(p, dst, a.x0, a.j0, lane, 0, uin, u0, Tin);
+    } else if (n == 1) {
+        if (lane < a.h)
+            res_ghosts<S, C, NV, TH, 1, OUT>(p, dst, a.x0, a.j0, lane, a.w - 1, C(0), C(0), C(0));
+    } else if (c < a.w) {
+        if (n < 4)
+            res_ghosts<S, C, NV, TH, 2, OUT>(p, dst, a.x0, a.j0, 0, c, C(0), C(0), C(0));
+        else
+            res_ghosts<S, C, NV, TH, 3, OUT>(p, dst, a.x0, a.j0, a.h - 1, c, C(0), C(0), C(0));
+    }
 }
 
 // All steps of one tile.  RPW: rows per warp.  Returns false when a wait ran out.
@@ -541,7 +592,7 @@ __device__ __forceinline__ bool res_tile(const StepParams<C> &p, const ResCtl &c
     const bool alone = ctl.ns * ctl.nb == 1;
     const float2 *stab = nullptr;
     if (threadIdx.x == 0)
-        t.nsend() = 0;
+        t.nsend() = t.taken() = 0;
     if constexpr (std::is_same<C, float>::value) {
         if (p.ntab > 1 && p.ntab <= SMEM_TAB) {
             load_smem_table(p, t.tab());
@@ -582,6 +633,8 @@ __device__ __forceinline__ bool res_tile(const StepParams<C> &p, const ResCtl &c
             ok = res_receive<C, NV, TH>(p, ctl.spin_limit, ctl.box + (seq & 1u) * half_words + own * words, seq);
         if (__syncthreads_or(!ok))
             return false;
+        if (threadIdx.x == 0)
+            t.taken() = 0;  // (read again only after the next barrier)
 
         // phase 1: pull, moments
         V f[RPW][9], g[RPW][4];
@@ -727,20 +780,21 @@ __device__ __forceinline__ bool res_tile(const StepParams<C> &p, const ResCtl &c
         if (send)
             res_send<C, NV, TH, RPW>(half, a, own, ctl.ns, warp * RPW, below, above, left, right, seq + 1);
         if (!left || !right || !below || !above) {
-            // the lattice's edge nodes fill the ghosts: a warp per edge (the first of a pair has
-            // all of a one-column or one-row lattice)
-            __syncthreads();
-            S *out = last ? dst : nullptr;
-            for (int n = warp; n < 4; n += warps) {
-                if (n == 0 ? left : (n == 1 ? right || p.nx == 1 : (n == 2 ? below : above || p.nr == 1)))
+            // the lattice's edge nodes fill the ghosts, a warp per task; the others do not wait
+            auto task = [&](int n) {
+                return n == 0 ? !left : (n == 1 ? !right : (n < 4 ? !below : !above) && 32 * (n & 1) < a.w);
+            };
+            bool mine = false;
+            for (int n = warp; n < RES_EDGES; n += warps)
+                mine = mine || task(n);
+            named_barrier(1, mine);
+            for (int n = warp; n < RES_EDGES; n += warps) {
+                if (!task(n))
                     continue;
-                if (n < 2) {
-                    if (lane < a.h)
-                        res_ghosts<S, C, NV, TH, 2>(p, out, a.x0, a.j0, lane, n ? a.w - 1 : 0, uin, u0, Tin);
-                } else {
-                    for (int c = lane; c < a.w; c += 32)
-                        res_ghosts<S, C, NV, TH, 1>(p, out, a.x0, a.j0, n == 2 ? 0 : a.h - 1, c, C(0), C(0), C(0));
-                }
+                if (last)
+                    res_edge_task<S, C, NV, TH, true>(p, dst, a, n, uin, u0, Tin);
+                else
+                    res_edge_task<S, C, NV, TH, false>(p, dst, a, n, uin, u0, Tin);
                 if (send)
                     res_send_corners<C, NV, TH>(half, t, 64 + n, seq + 1);
             }
