@@ -538,7 +538,8 @@ __device__ __noinline__ void res_ghosts(const StepParams<C> &p, S *dst, const in
                     M.j(o) = make_float2(gx, gr);
                     M.T(o) = gT;
                 }
-                s = store_as<S, C>(edge_sub<C>(p, q, gx, gr, gT, v));
+                // (write_ghosts' rounding: beyond the axis as in a collision's store)
+                s = store_as<S, C>(SIDE == 2 ? split_sub<C>(p, q, gx, gr, gT, v) : edge_sub<C>(p, q, gx, gr, gT, v));
                 v = split_add<C>(p, q, gx, gr, gT, load_as_shared<S, C>(&s));
             }
         } else {

@@ -72,6 +72,34 @@ def test_the_largest_tiles_and_the_first_lattices_beyond_them(lbm, storage, size
     same(one, many)
 
 
+@pytest.mark.parametrize("storage", ["f16s", "bf16s"])
+@pytest.mark.parametrize("bounds", ["jet", "substrate", "pipe"])
+def test_smooth_flows_of_the_moment_split_types_equal_single_steps(lbm, bounds, storage):
+    """Where the deviations are small, one FP32 rounding of a ghost cell's linear part shows: a
+    hot smooth flow, quiet at the axis, over many nodes and steps."""
+    nx, nr = 2000, 48
+    x, r = torch.arange(nx).double()[None] / nx, (torch.arange(nr).double()[:, None] + 0.5) / nr
+    for seed in range(6):
+        one, many = pair(lbm, nx, nr, storage, bounds, seed)
+        gen = torch.Generator().manual_seed(seed)
+        a = torch.rand(4, generator=gen).double()
+        ux = 0.03 + 0.02 * torch.sin(5 * x + 6 * a[0]) * torch.cos(3 * r)
+        ur = 0.01 * r * torch.cos(7 * x + 6 * a[1]) * (1 - r)
+        T = 1 + (5 + 5 * a[2]) * (1 - 0.6 * x) * torch.exp(-3 * r * r)
+        w9 = [4 / 9] + [1 / 9] * 4 + [1 / 36] * 4
+        e9 = [(0, 0), (1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1)]
+        f = torch.stack([w * (1 + 3 * (ux * c + ur * d) + 4.5 * (ux * c + ur * d) ** 2 - 1.5 * (ux ** 2 + ur ** 2))
+                         for w, (c, d) in zip(w9, e9)])
+        g = torch.stack([0.25 * T * (1 + 2 * (ux * c + ur * d)) for c, d in e9[1:5]])
+        g = g * (1 + 4e-4 * (torch.rand(g.shape, generator=gen).double() - 0.5))
+        one.set_state(f.cuda(), g.cuda(), 0)
+        many.set_state(f.cuda(), g.cuda(), 0)
+        for _ in range(120):
+            one.step(1)
+        many.step(120)
+        same(one, many)
+
+
 def test_lattices_on_two_streams(lbm):
     lats = [pair(lbm, 500, 120, "f32", "jet", seed=7 + k) for k in range(4)]
     streams = [torch.cuda.Stream() for _ in lats]
