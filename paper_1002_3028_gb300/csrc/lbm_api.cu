@@ -459,16 +459,18 @@ int plan_launch(lbm_lattice *h)
 }
 
 // Lattices that fit the chip run their steps there (lbm_resident.cuh): strips of 64 columns
-// (FP64 32), cut into tiles of one CTA each, every CTA resident.  Of the tile shapes, in FP32
-// arithmetic: eight rows, one a warp, while one tile a SM is enough (us per step: 200 x 96
-// FP32 3.4 with tiles of 8 rows; 0.4 more in tiles of 6, 0.7 of 4, 2.3 of 16 rows with two
-// rows a warp);
-// then the same with two CTAs a SM, whose registers leave room for six warps each
-// (640 x 160 FP16 moment-split 4.5 in tiles of 5 and 6 rows, 1.0 more of 14 with two rows a
-// warp); then sixteen rows, two a warp, two CTAs a SM (1024 x 256 FP32 6.0).  FP64 is bound by its
-// arithmetic: the tiles that spread it over the SMs best.  The step kernel takes 8.8, 15.8
-// and 12.4 us on the three lattices and keeps those that do not fit, those with periodic
-// ends or in the AA layout, and those whose launch shape the caller has set.
+// (32 with one node a lane), cut into tiles of one CTA each, every CTA resident.  A step's
+// time is what one tile's takes, so the lattice is spread as far as its tiles stay worth
+// their rings; of the tile shapes, in this order (FP32 arithmetic; us per step):
+//   32 x 8, a row a warp, one tile a SM    200 x 96 FP32 3.0 (64 x 8: 3.4; the step kernel 8.8)
+//   64 x 8, a row a warp, one tile a SM    512 x 128 FP32 3.4 (64 x 16: 3.9; 10.3)
+//   the same with two CTAs a SM, whose registers leave room for six warps each
+//                                          640 x 160 FP16 moment-split 4.4 (64 x 11: 4.6; 15.8)
+//   64 x 16, a row a warp, one tile a SM   900 x 140 FP32 4.3 (two rows a warp: 5.1 to 5.9; 11.5)
+//   64 x 16, two rows a warp, two a SM     1024 x 256 FP32 6.0 (12.4)
+// FP64 is bound by its arithmetic: the tiles that spread it over the SMs best.  The step
+// kernel keeps lattices that do not fit, those with periodic ends or in the AA layout, and
+// those whose launch shape the caller has set.
 cudaError_t res_occupancy(const lbm_lattice *h, int shape, int warps, int *per_sm)
 {
     switch (h->d.storage) {
@@ -489,7 +491,7 @@ void res_plan(lbm_lattice *h)
         h->nv != default_nv(d.storage))
         return;
     auto fits = [&](int shape, int nb) {
-        const int W = strip_cols(d.storage);
+        const int W = 32 * lbm::res_nv(shape, default_nv(d.storage));
         const int ns = (d.nx + W - 1) / W;
         const int rows = (d.nr + nb - 1) / nb;
         if (nb < 1 || rows > lbm::res_rows(shape) || (nb > 1 && d.nr / nb < 2) || (ns > 1 && d.nx / ns < 2))
@@ -513,7 +515,8 @@ void res_plan(lbm_lattice *h)
     if (d.storage == LBM_F64)
         (void)(fits(0, up(cols, one, 4)) || fits(0, up(cols, two, 4)) || fits(2, up(cols, one, 4)));
     else
-        (void)(fits(0, up(cols, one, 8)) || fits(0, up(cols, two, 4)) || fits(1, up(cols, two, 4)));
+        (void)(fits(3, up(32, one, 8)) || fits(0, up(cols, one, 8)) || fits(0, up(cols, two, 4)) ||
+               fits(2, up(cols, one, 8)) || fits(1, up(cols, two, 4)));
 }
 
 cudaError_t res_launch(lbm_lattice *h, const lbm::ResCtl &ctl, const ResPlan &r, cudaStream_t s)
@@ -578,7 +581,10 @@ int res_ready(lbm_lattice *h, const ResPlan &r, bool capturing, cudaStream_t s, 
     return LBM_OK;
 }
 
-constexpr int kResMinSteps = 2;  // one step reads and writes the lattice once either way
+// steps from which a call is worth the load of the tiles and their rings (us for 2 steps, the
+// step kernel against this: 64 x 32 FP32 17 and 15, 1024 x 256 FP32 29 and 27; FP64
+// 64 x 32 40 and 44, for 6 steps 101 and 101)
+int res_min_steps(int storage) { return storage == LBM_F64 ? 6 : 2; }
 
 // *done: steps taken (fewer than nsteps when the tiles cannot all be resident after all)
 int res_step(lbm_lattice *h, const ResPlan &r, int nsteps, bool capturing, cudaStream_t s, int *done)
@@ -1282,7 +1288,7 @@ static int step_impl(lbm_lattice *h, int32_t nsteps, lbm_stream stream)
         return cuda_fail(cudaGetLastError(), "querying the stream");
     if (cap != cudaStreamCaptureStatusNone)
         h->sync_captured = true;
-    if (nsteps >= kResMinSteps && h->res.shape >= 0) {
+    if (nsteps >= res_min_steps(d.storage) && h->res.shape >= 0) {
         int done = 0;
         const int rc = res_step(h, h->res, nsteps, cap != cudaStreamCaptureStatusNone, s, &done);
         if (rc)

@@ -359,6 +359,32 @@ __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(__fmul2_rn(a.v, 
 __device__ __forceinline__ F2 operator-(F2 a) { return F2(make_float2(-a.v.x, -a.v.y)); }
 __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 
+// Vec<float, -1>: one node, by the paired instructions (the second half of a pair is left
+// undefined), for kernels whose one node a lane has to have the bits of two: ptxas may fuse a
+// scalar product with a power of two into the sum that follows, which differs from the paired
+// sequence where the product underflows.
+template <>
+struct Vec<float, -1> {
+    float x;
+    __device__ __forceinline__ Vec() {}
+    __device__ __forceinline__ explicit Vec(float s) : x(s) {}
+    __device__ __forceinline__ float operator[](int) const { return x; }
+    __device__ __forceinline__ void set(int, float v) { x = v; }
+    __device__ __forceinline__ float2 pair() const
+    {
+        float2 p;
+        p.x = x;
+        return p;
+    }
+};
+using F1 = Vec<float, -1>;
+__device__ __forceinline__ F1 operator+(F1 a, F1 b) { return F1(__fadd2_rn(a.pair(), b.pair()).x); }
+__device__ __forceinline__ F1 operator-(F1 a, F1 b) { return F1(__ffma2_rn(b.pair(), F1(-1.f).pair(), a.pair()).x); }
+__device__ __forceinline__ F1 operator*(F1 a, F1 b) { return F1(__fmul2_rn(a.pair(), b.pair()).x); }
+__device__ __forceinline__ F1 operator-(F1 a) { return F1(-a.x); }
+__device__ __forceinline__ F1 vfma(F1 a, F1 b, F1 c) { return F1(__ffma2_rn(a.pair(), b.pair(), c.pair()).x); }
+__host__ __device__ constexpr int vec_nodes(int n) { return n < 0 ? 1 : n; }
+
 template <class C, int N> __device__ __forceinline__ Vec<C, N> operator*(C s, Vec<C, N> a) { return Vec<C, N>(s) * a; }
 template <class C, int N> __device__ __forceinline__ Vec<C, N> operator+(C s, Vec<C, N> a) { return Vec<C, N>(s) + a; }
 template <class C, int N> __device__ __forceinline__ Vec<C, N> operator-(Vec<C, N> a, C s) { return a - Vec<C, N>(s); }
@@ -370,7 +396,7 @@ __device__ __forceinline__ Vec<C, N> vrcp(Vec<C, N> a)
 {
     Vec<C, N> r;
 #pragma unroll
-    for (int c = 0; c < N; ++c)
+    for (int c = 0; c < vec_nodes(N); ++c)
         r.set(c, C(1) / a[c]);
     return r;
 }
@@ -380,7 +406,7 @@ __device__ __forceinline__ Vec<C, N> vsqrt(Vec<C, N> a)
 {
     Vec<C, N> r;
 #pragma unroll
-    for (int c = 0; c < N; ++c)
+    for (int c = 0; c < vec_nodes(N); ++c)
         r.set(c, sqrt(a[c]));
     return r;
 }

@@ -20,9 +20,9 @@
 // release and the neighbours' acquire.  Here a step is two barriers, one
 // collision's latency per row a warp holds, and the exchange of the ring.
 // us per step, the step kernel against this one (200 steps a launch):
-// 64 x 32 FP32 6.7 -> 3.3, 200 x 96 FP32 8.8 -> 3.4 and FP64 19.5 -> 16.2,
-// 640 x 160 FP16 moment-split 15.8 -> 4.5, 777 x 301 17.9 -> 7.6,
-// 1024 x 256 FP32 12.4 -> 6.0.  With the exchange's waits taken out the last
+// 64 x 32 FP32 6.6 -> 3.0, 200 x 96 FP32 8.6 -> 3.0 and FP64 19.4 -> 16.1,
+// 900 x 140 FP32 11.5 -> 4.4, 640 x 160 FP16 moment-split 15.2 -> 4.4,
+// 1024 x 256 16.2 -> 7.3 and FP32 12.5 -> 6.0.  With the exchange's waits taken out the last
 // takes 4.6: the rest is the way of a value through L2 and the slowest tile
 // of each neighbourhood, one at a lattice edge, whose ghosts come after its
 // collisions.
@@ -76,9 +76,10 @@ struct ResTile {
     }
 };
 
-// tile shapes: the most rows of a tile and the rows a warp holds (2: FP64 only)
-constexpr int RES_SHAPES = 3;
-__host__ __device__ constexpr int res_rows(int shape) { return shape == 0 ? 8 : 16; }
+// tile shapes: the most rows of a tile, the rows a warp holds and the nodes a lane holds of a
+// row (at most `widest`: 2, in FP64 1; FP64 has shapes 0 and 2)
+__host__ __device__ constexpr int res_rows(int shape) { return shape == 0 || shape == 3 ? 8 : 16; }
+__host__ __device__ constexpr int res_nv(int shape, int widest) { return shape == 3 ? 1 : widest; }
 __host__ __device__ constexpr int res_rpw(int shape) { return shape == 1 ? 2 : 1; }
 
 constexpr int RES_CORNERS = 32;     // corner entries of an inbox (res_corner; two unused)
@@ -129,7 +130,7 @@ constexpr int RES_NONE = 0xffff;
 // 8-byte words of a tile's inbox
 __host__ __device__ constexpr int64_t res_box_words(int value_bytes, int shape)
 {
-    return (int64_t)(24 * 32 * (value_bytes == 8 ? 1 : 2) + 16 * res_rows(shape) + RES_CORNERS) *
+    return (int64_t)(24 * 32 * res_nv(shape, value_bytes == 8 ? 1 : 2) + 16 * res_rows(shape) + RES_CORNERS) *
            (value_bytes / 4);
 }
 
@@ -585,7 +586,8 @@ __device__ __forceinline__ void res_edge_task(const StepParams<C> &p, S *dst, co
 template <class S, class C, int NV, int TH, int RPW>
 __device__ __forceinline__ bool res_tile(const StepParams<C> &p, const ResCtl &ctl, const ResTile &a)
 {
-    using V = Vec<C, NV>;
+    // (one FP32 node a lane by the instructions of two, so that every tile shape gives the same bits)
+    using V = Vec<C, NV == 1 && std::is_same<C, float>::value ? -1 : NV>;
     using Mem = ResMem<C, NV, TH>;
     const Mem t;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;

@@ -124,11 +124,10 @@ cudaError_t LBM_CAT(occupancy_batch_, LBM_TAG)(int warps_per_cta, int nv, int *c
 }
 
 // resident lattices (lbm_resident.cuh): one CTA per tile, all of them resident at once.
-// Two rows a warp in FP32 arithmetic, one in FP64, fill tiles of sixteen rows.
 template <int SHAPE>
 static void res_instance(const void **fn, int *smem)
 {
-    constexpr int NV = LBM_MAX_NV;
+    constexpr int NV = res_nv(SHAPE, LBM_MAX_NV);
     *fn = reinterpret_cast<const void *>(res_run_kernel<LBM_S, LBM_C, NV, res_rows(SHAPE), res_rpw(SHAPE)>);
     *smem = res_smem<LBM_S, LBM_C, NV, res_rows(SHAPE)>();
 }
@@ -139,12 +138,13 @@ static const void *res_kernel(int shape, int *smem)
     *smem = 0;
     if (shape == 0)
         res_instance<0>(&fn, smem);
+    if (shape == 2)
+        res_instance<2>(&fn, smem);
 #if LBM_MAX_NV > 1
     if (shape == 1)
         res_instance<1>(&fn, smem);
-#else
-    if (shape == 2)
-        res_instance<2>(&fn, smem);
+    if (shape == 3)
+        res_instance<3>(&fn, smem);
 #endif
     return fn;
 }
