@@ -255,7 +255,7 @@ __device__ __forceinline__ bool ghost_moments(const StepParams<C> &p, int ci, in
 }
 
 template <class C>
-__device__ __forceinline__ int64_t cell(const StepParams<C> &p, int q, int i, int j)
+__host__ __device__ __forceinline__ int64_t cell(const StepParams<C> &p, int q, int i, int j)
 {
     return (int64_t)q * p.plane + (int64_t)(j + 1) * p.pitch + (i + PAD_COLS);
 }
@@ -639,7 +639,7 @@ __device__ __noinline__ void write_ghosts(const StepParams<C> &p, S *buf, int i,
 // state: the post-collision value of node (i, j) - e_q (two buffers), or
 // the AA layout's slot for that population in the state's representation
 template <class C>
-__device__ __forceinline__ int64_t stream_cell(const StepParams<C> &p, int q, int i, int j)
+__host__ __device__ __forceinline__ int64_t stream_cell(const StepParams<C> &p, int q, int i, int j)
 {
     if (p.aa && p.phase)
         return cell(p, q, i, j);
@@ -1699,23 +1699,6 @@ __global__ void fill_ghosts_kernel(const __grid_constant__ StepParams<C> p)
     const int n = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (n < edge_nodes(p.nx, p.nr) && edge_node(p.nx, p.nr, n, i, j))
         write_ghosts<S, C>(p, static_cast<S *>(p.dst), i, j, p.step);
-}
-
-// ---- fields at the current time: Eq. 2 moments of the streamed populations ---------------
-template <class S, class C, class O>
-__global__ void fields_kernel(const __grid_constant__ StepParams<C> p, O *out)
-{
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t N = (int64_t)p.nx * p.nr;
-    if (n >= N)
-        return;
-    const int i = (int)(n % p.nx), j = (int)(n / p.nx);
-    const Mom<Vec<C, 1>> m = node_moments<S, C>(p, i, j, false);
-    const C rho = p.rho0 + m.drho.x;
-    out[n] = O(rho);
-    out[N + n] = O(m.jx.x / rho);
-    out[2 * N + n] = O(m.jr.x / rho);
-    out[3 * N + n] = O(p.T0 + m.dT.x);
 }
 
 // ---- FP64 diagnostics: mass, heat, steady residual, divergence -------------------------

@@ -156,6 +156,94 @@ inline unsigned read_blocks(int rows, int nx)
     return (unsigned)((items + 7) / 8);
 }
 
+// ---- fields at the current time: Eq. 2 moments of the streamed populations ---------------
+// element offsets of the populations streamed into node (0, 0) (stream_cell)
+template <class C>
+__host__ __device__ inline PlaneOffsets stream_planes(const StepParams<C> &p)
+{
+    PlaneOffsets o;
+    for (int q = 0; q < 13; ++q)
+        o.off[q] = stream_cell(p, q, 0, 0);
+    return o;
+}
+
+__device__ __forceinline__ void put_field(float *o, float v) { *o = v; }
+__device__ __forceinline__ void put_field(float *o, double v) { *o = (float)v; }
+__device__ __forceinline__ void put_field(double *o, double v) { *o = v; }
+__device__ __forceinline__ void put_field(double *o, float v)
+{
+    *o = (__float_as_uint(v) << 1) == 0 ? __hiloint2double((int)__float_as_uint(v), 0) : diag_double(v);
+}
+
+// moment-split storage: a thermal population from its deviation, as the linear part's sum rounds
+// when it is formed before the deviation is added
+template <class C>
+__device__ __forceinline__ C field_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d)
+{
+    const C x = rn_mul(rn_add(p.T0, dT), p.hir0);
+    return rn_add(d, rn_fma(C(0.25), dT, rn_mul(x, edot<C>(ex4(q - 9), ey4(q - 9), jx, jr))));
+}
+
+// A node a lane, all of its loads in flight together; a CTA takes 32 columns by eight rows, so
+// that the moments of moment-split storage, which the nodes of three rows read, come from L1.
+// Bound by memory in FP32.  4096 x 1024 into FP64 / FP32 fields, us, before (a node a thread in
+// row order, its position by 64-bit division, the moments again for each population, past L1) ->
+// now, and the bytes at the copy rate: FP32 56 / 50 -> 54 / 44 (53 / 43), FP16 49 / 40 -> 45 / 35
+// (36 / 26), FP16 moment-split 102 / 99 -> 62 / 50 (44 / 34).  Two nodes a lane: 54 / 44, 47 / 37
+// and 77 / 57.
+template <class S, class C, class O>
+__global__ void __launch_bounds__(256) fields_kernel(const __grid_constant__ StepParams<C> p,
+                                                     const __grid_constant__ PlaneOffsets planes, O *out)
+{
+    const unsigned pieces = (unsigned)(p.nx + 31) / 32, group = blockIdx.x / pieces;
+    const int i = (int)(32 * (blockIdx.x - group * pieces) + (threadIdx.x & 31)), j = (int)(8 * group + (threadIdx.x >> 5));
+    if (j >= p.nr)
+        return;
+    const S *src = static_cast<const S *>(p.src) + (int64_t)j * p.pitch;
+    Vec<C, 1> f[9], g[4];
+    float2 jj[9];
+    float T[4];
+    if (i < p.nx) {
+        if constexpr (IsSplit<S>::value) {  // the moments of the nodes around
+            const float *M = split_m(static_cast<const S *>(p.src), p.plane);
+            const int64_t o = cell(p, 0, i, j);
+#pragma unroll
+            for (int q = 1; q < 9; ++q) {
+                const int64_t s = o - ey9(q) * p.pitch - ex9(q);
+                jj[q] = __ldg(reinterpret_cast<const float2 *>(M) + s);
+                if (q < 5)
+                    T[q - 1] = __ldg(M + 2 * p.plane + s);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+            f[q].x = load_as<S, C>(src + planes.off[q] + i);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            g[q].x = load_as<S, C>(src + planes.off[9 + q] + i);
+    }
+    const int64_t N = (int64_t)p.nx * p.nr;
+    out += (int64_t)j * p.nx;
+    // (a branch between the loads and their use keeps all of them in flight: 48 registers for
+    // moment-split storage; without it 34, and 74 / 58 us)
+    if (i < p.nx) {
+        if constexpr (IsSplit<S>::value) {
+#pragma unroll
+            for (int q = 1; q < 9; ++q)
+                f[q].x = edge_add<C>(p, q, jj[q].x, jj[q].y, 0.f, f[q].x);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                g[q].x = field_add<C>(p, 9 + q, jj[q + 1].x, jj[q + 1].y, T[q], g[q].x);
+        }
+        const Mom<Vec<C, 1>> m = moments<Vec<C, 1>>(f, g);
+        const C rho = p.rho0 + m.drho.x;
+        put_field(out + i, rho);
+        put_field(out + N + i, m.jx.x / rho);
+        put_field(out + 2 * N + i, m.jr.x / rho);
+        put_field(out + 3 * N + i, p.T0 + m.dT.x);
+    }
+}
+
 // ---- checkpoints ---------------------------------------------------------------------
 // Rows of `planes` planes between the padded buffer and a dense [plane][row][n]
 // array, in words of type U.  One launch instead of a strided copy per plane

@@ -185,13 +185,12 @@ cudaError_t LBM_CAT(occupancy_res_, LBM_TAG)(int shape, int warps, int *ctas_per
 
 cudaError_t LBM_CAT(launch_fields_, LBM_TAG)(const StepParams<LBM_C> &p, void *out, int out_f64, cudaStream_t s)
 {
-    const int64_t N = (int64_t)p.nx * p.nr;
-    const int threads = 256;
-    const int64_t blocks = (N + threads - 1) / threads;
+    const unsigned blocks = (unsigned)((p.nx + 31) / 32) * (unsigned)((p.nr + 7) / 8);
+    const PlaneOffsets o = stream_planes(p);
     if (out_f64)
-        fields_kernel<LBM_S, LBM_C, double><<<(unsigned)blocks, threads, 0, s>>>(p, static_cast<double *>(out));
+        fields_kernel<LBM_S, LBM_C, double><<<blocks, 256, 0, s>>>(p, o, static_cast<double *>(out));
     else
-        fields_kernel<LBM_S, LBM_C, float><<<(unsigned)blocks, threads, 0, s>>>(p, static_cast<float *>(out));
+        fields_kernel<LBM_S, LBM_C, float><<<blocks, 256, 0, s>>>(p, o, static_cast<float *>(out));
     return cudaGetLastError();
 }
 

@@ -74,3 +74,26 @@ def test_checkpoints_of_every_row_alignment(lbm, nx, storage, pattern, steps):
     a.step(2)
     b.step(2)
     assert torch.equal(a.save()[0], b.save()[0])
+
+
+@pytest.mark.parametrize("storage,pattern,steps", [("f64", "ab", 1), ("f32", "ab", 1), ("bf16", "ab", 1), ("f16s", "ab", 1),
+                                                   ("f32", "aa", 1), ("f16", "aa", 2)])
+@pytest.mark.parametrize("size", [(3, 3), (33, 9), (64, 8), (65, 17), (258, 40)], ids=lambda s: f"{s[0]}x{s[1]}")
+def test_fields_are_the_moments_of_the_streamed_populations(lbm, size, storage, pattern, steps):
+    """Inside the lattice, where every population comes from a node of the state."""
+    nx, nr = size
+    lat = lbm.Lattice.from_workload(I.jet_workload(nx=nx, nr=nr), storage, device="cuda:0", pattern=pattern)
+    lat.step(steps)
+    f, g = lat.get_state()
+    e9 = [(0, 0), (1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1)]
+    pull = lambda p, e: torch.roll(p, (e[1], e[0]), (0, 1))
+    f, g = [pull(p, e) for p, e in zip(f, e9)], [pull(p, e) for p, e in zip(g, e9[1:5])]
+    rho = sum(f)
+    want = torch.stack([rho, sum(p * e[0] for p, e in zip(f, e9)) / rho, sum(p * e[1] for p, e in zip(f, e9)) / rho, sum(g)])
+    inside = (slice(None), slice(1, -1), slice(1, -1))
+    eps = 2.0 ** -53 if storage == "f64" else 2.0 ** -24
+    scale = max(1.0, float(want.abs().max()))
+    for dtype in (torch.float64, torch.float32):
+        got = lat.fields(dtype=dtype).double()
+        # 13 terms of at most the largest value, each sum rounded once, and the quotient's
+        assert (got - want)[inside].abs().max() <= 16 * (eps if dtype == torch.float64 else max(eps, 2.0 ** -24)) * scale
