@@ -582,8 +582,8 @@ int res_ready(lbm_lattice *h, const ResPlan &r, bool capturing, cudaStream_t s, 
 }
 
 // steps from which a call is worth the load of the tiles and their rings (us for 2 steps, the
-// step kernel against this: 64 x 32 FP32 17 and 15, 1024 x 256 FP32 29 and 27; FP64
-// 64 x 32 40 and 44, for 6 steps 101 and 101)
+// step kernel against this: 64 x 32 FP32 17 and 13, 1024 x 256 FP32 28 and 25; FP64
+// 64 x 32 40 and 44, for 6 steps 98 and 98, 200 x 96 130 and 105)
 int res_min_steps(int storage) { return storage == LBM_F64 ? 6 : 2; }
 
 // *done: steps taken (fewer than nsteps when the tiles cannot all be resident after all)
