@@ -1729,11 +1729,21 @@ __device__ __forceinline__ double diag_max(double a, double b)  // a, or b if it
     const long long m = __double_as_longlong(b);
     return m > __double_as_longlong(a) && m <= 0x7ff0000000000000ll ? b : a;
 }
-__device__ __forceinline__ double diag_rcp(double a)
+__device__ __forceinline__ bool diag_finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+// (ux, ur) = (jx, jr) / rho.  A density that FP32 cannot hold with room to spare, and one that is not positive, takes
+// the FP64 division.
+__device__ __forceinline__ void diag_velocity(double jx, double jr, double rho, double &ux, double &ur)
 {
-    double y = (double)(1.f / (float)a);
-    y = fma(y, fma(-a, y, 1.0), y);
-    return fma(y, fma(-a, y, 1.0), y);
+    if ((unsigned)__double2hiint(rho) - ((1023u - 100u) << 20) < 200u << 20) {
+        double y = (double)(1.f / (float)rho);
+        y = fma(y, fma(-rho, y, 1.0), y);
+        y = fma(y, fma(-rho, y, 1.0), y);
+        ux = jx * y;
+        ur = jr * y;
+    } else {
+        ux = jx / rho;
+        ur = jr / rho;
+    }
 }
 
 __device__ __forceinline__ double diag_combine(int k, double a, double b)
@@ -1770,12 +1780,12 @@ __device__ __forceinline__ void diag_node(const StepParams<C> &p, int have_prev,
     const Mom<Vec<C, 1>> m = node_moments<S, C>(p, i, j, false);
     const double rho = diag_double(p.rho0) + diag_double(m.drho.x);
     const double T = diag_double(p.T0) + diag_double(m.dT.x);
-    const double jx = diag_double(m.jx.x), jr = diag_double(m.jr.x);
-    if (!(rho > 0.0) || !isfinite(rho) || !isfinite(T) || !isfinite(jx) || !isfinite(jr)) {
+    double ux, ur;
+    diag_velocity(diag_double(m.jx.x), diag_double(m.jr.x), rho, ux, ur);
+    if (!(rho > 0.0) || !diag_finite(rho) || !diag_finite(T) || !diag_finite(ux) || !diag_finite(ur)) {
         v[7] += 1.0;
         return;
     }
-    const double inv = diag_rcp(rho), ux = jx * inv, ur = jr * inv;
     const double r = diag_double(p.r0) + j + 0.5;
     v[0] += rho;
     v[1] += r * rho;
@@ -1786,8 +1796,9 @@ __device__ __forceinline__ void diag_node(const StepParams<C> &p, int have_prev,
     v[6] = diag_max(v[6], uu);
     if (have_prev) {
         const Mom<Vec<C, 1>> q = node_moments<S, C>(p, i, j, true);
-        const double ip = diag_rcp(diag_double(p.rho0) + diag_double(q.drho.x));
-        const double dx = ux - diag_double(q.jx.x) * ip, dr = ur - diag_double(q.jr.x) * ip;
+        double px, pr;
+        diag_velocity(diag_double(q.jx.x), diag_double(q.jr.x), diag_double(p.rho0) + diag_double(q.drho.x), px, pr);
+        const double dx = ux - px, dr = ur - pr;
         const double dd = dx * dx + dr * dr;
         v[4] += dd;
         v[5] = diag_max(v[5], dd);
