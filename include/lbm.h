@@ -305,7 +305,7 @@ LBM_API int lbm_set_state(lbm_lattice *h, const double *dev_f, const double *dev
  * lbm_save: copy the stored post-collision populations, as deviations
  *   from rest (f_k - w_k rho0 and g_k - T0 / 4, in the storage type; the
  *   same values and layout for both patterns), into dev_out,
- *   caller device memory of lbm_checkpoint_bytes bytes, layout
+ *   caller device memory of lbm_checkpoint_bytes bytes at any address, layout
  *   [q][j][i] with q = f0..f8, g0..g3.  The step counter is read with
  *   lbm_get_step.  Asynchronous on the stream.
  * lbm_restore: the reverse, into a lattice of the same size and storage

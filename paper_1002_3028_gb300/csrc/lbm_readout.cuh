@@ -308,7 +308,9 @@ inline cudaError_t plane_copy(void *padded, void *dense, int planes, int64_t row
         return plane_copy_as<uint2>(padded, dense, planes, row_bytes, nr, pitch_bytes, byte_offs, out, s);
     if (a % 4 == 0)
         return plane_copy_as<unsigned>(padded, dense, planes, row_bytes, nr, pitch_bytes, byte_offs, out, s);
-    return plane_copy_as<unsigned short>(padded, dense, planes, row_bytes, nr, pitch_bytes, byte_offs, out, s);
+    if (a % 2 == 0)
+        return plane_copy_as<unsigned short>(padded, dense, planes, row_bytes, nr, pitch_bytes, byte_offs, out, s);
+    return plane_copy_as<unsigned char>(padded, dense, planes, row_bytes, nr, pitch_bytes, byte_offs, out, s);
 }
 
 }  // namespace lbm
