@@ -453,7 +453,7 @@ __device__ bool wait_edges(const StepParams<C> &p, const unsigned *pub, int cols
             __syncwarp();  // every lane now sees what its watcher acquired
             return true;
         }
-        if (it >= spin_limit || (*static_cast<volatile int *>(p.status) & STATUS_TIMEOUT))
+        if (it >= spin_limit || wait_given_up(p.status))
             return false;
         __nanosleep(it < 32 ? 32 : (it < 128 ? 256 : 2048));  // these waits are short: poll finely first
     }

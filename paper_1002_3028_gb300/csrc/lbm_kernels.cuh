@@ -1471,6 +1471,14 @@ __device__ __forceinline__ void red_release_add(unsigned *a, unsigned v)
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;\n" ::"l"(a), "r"(v) : "memory");
 }
 
+// Whether a wait ran out somewhere in the launch.  All lanes of the calling warp get the same
+// answer, so that a warp gives up its wait as a whole: a lane that left alone would leave the
+// others in the next vote for good.
+__device__ __forceinline__ bool wait_given_up(const int *status)
+{
+    return __any_sync(0xffffffffu, *static_cast<const volatile int *>(status) & STATUS_TIMEOUT);
+}
+
 // Every lane waits until the items around item (band b, column g) of a
 // lattice (its counters start at `flags`, `cols` items per band, each at
 // `base` before sub-step 0) have
@@ -1508,7 +1516,7 @@ __device__ bool wait_neighbours(const StepParams<C> &p, const unsigned *flags, i
             __syncwarp();  // orders memory among the lanes: every lane now sees what its watcher acquired
             return true;
         }
-        if (it >= spin_limit || (*static_cast<volatile int *>(p.status) & STATUS_TIMEOUT))
+        if (it >= spin_limit || wait_given_up(p.status))
             return false;
         __nanosleep(it < 8 ? 64 : (it < 64 ? 512 : 2048));
     }

@@ -291,11 +291,12 @@ __device__ __noinline__ void res_lists(const StepParams<C> &p, const int ns, con
 }
 
 // ---- receiving ---------------------------------------------------------------------------
-// one more poll of a wait?  Sleeps between polls; false when the wait runs out or another's did.
+// one more poll of a wait?  Sleeps between polls; false, in the whole warp, when the wait runs out or
+// another's did.
 template <class C>
 __device__ __forceinline__ bool res_poll_again(const StepParams<C> &p, int spin_limit, int it)
 {
-    if (it >= spin_limit || (it > 64 && (*static_cast<volatile int *>(p.status) & STATUS_TIMEOUT)))
+    if (it >= spin_limit || (it > 64 && wait_given_up(p.status)))
         return false;
     if (it > 32)
         __nanosleep(it < 256 ? 32 : 1024);
