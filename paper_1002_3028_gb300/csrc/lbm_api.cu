@@ -519,6 +519,38 @@ void res_plan(lbm_lattice *h)
                fits(2, up(cols, one, 8)) || fits(1, up(cols, two, 4)));
 }
 
+// Allocations and releases within: another thread's capture of a graph goes on (its mode may
+// forbid them to every thread).
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Releases the inboxes after the lattice's last use, on a stream that orders nothing else (the
+// default stream would hold up the caller's work on it until then).
+void res_release(lbm_lattice *h)
+{
+    if (!h->res_box)
+        return;
+    const RelaxedCapture relaxed;
+    int device = h->device;
+    cudaGetDevice(&device);
+    if (device != h->device)
+        cudaSetDevice(h->device);
+    cudaStream_t s = nullptr;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess)
+        s = nullptr;
+    cudaStreamWaitEvent(s, h->last, 0);
+    cudaFreeAsync(h->res_box, s);
+    if (s)
+        cudaStreamDestroy(s);  // once its work has run
+    if (device != h->device)
+        cudaSetDevice(device);
+    cudaGetLastError();
+    h->res_box = nullptr;
+}
+
 cudaError_t res_launch(lbm_lattice *h, const lbm::ResCtl &ctl, const ResPlan &r, cudaStream_t s)
 {
     switch (h->d.storage) {
@@ -563,6 +595,7 @@ int res_ready(lbm_lattice *h, const ResPlan &r, bool capturing, cudaStream_t s, 
         h->res_box = nullptr;
         h->res_bytes = 0;
         h->res_key = 0;
+        const RelaxedCapture relaxed;
         if (cudaMallocAsync(&h->res_box, bytes, s) != cudaSuccess) {
             cudaGetLastError();
             h->res_box = nullptr;
@@ -1189,10 +1222,7 @@ void lbm_destroy(lbm_lattice *h)
         cudaStreamWaitEvent(nullptr, h->last, 0);
         cudaFreeAsync(h->mem, nullptr);
     }
-    if (h->res_box) {
-        cudaStreamWaitEvent(nullptr, h->last, 0);
-        cudaFreeAsync(h->res_box, nullptr);
-    }
+    res_release(h);
     h->mem = nullptr;
     cudaEventDestroy(h->ready);
     cudaEventDestroy(h->last);
