@@ -205,6 +205,24 @@ LBM_API int lbm_set_properties(lbm_lattice *h, const double *nu, const double *a
  */
 LBM_API int lbm_step(lbm_lattice *h, int32_t nsteps, lbm_stream stream);
 
+/*
+ * How lbm_step keeps a lattice on the chip (any launch shape set since included): tiles of at
+ * most tile_cols x tile_rows nodes, tiles_across x tiles_up of them, rows_per_warp rows a warp;
+ * all 0 for a lattice that the step kernel runs.  min_steps: the steps from which a call runs
+ * there.  inbox_bytes: the device memory that the first such call allocates beside the memory of
+ * lbm_required_bytes (0 for a single tile); inbox_held: what is allocated now.  steps: the steps
+ * that have run there since lbm_create (fewer than were asked for where the inboxes could not
+ * be allocated: the step kernel took those).
+ */
+typedef struct {
+    int32_t tile_cols, tile_rows, rows_per_warp;
+    int32_t tiles_across, tiles_up;
+    int32_t min_steps;
+    int64_t inbox_bytes, inbox_held;
+    int64_t steps;
+} lbm_resident;
+LBM_API int lbm_get_resident(const lbm_lattice *h, lbm_resident *out);
+
 /* Number of steps taken so far (the time index of the inlet noise). */
 LBM_API int64_t lbm_get_step(const lbm_lattice *h);
 
@@ -261,7 +279,7 @@ LBM_API int lbm_check(lbm_lattice *h, int32_t *flags);
 
 /*
  * Self-test of the bounded waits of the persistent step launch (either
- * pattern's; no counterpart in the paper).  Runs one launch on the default stream in
+ * pattern's; no counterpart in the paper).  Runs a launch on the default stream in
  * which every work item waits for neighbours of a step that never runs,
  * with a wait limit of a few tens of microseconds: each wait gives up,
  * raises LBM_STATUS_TIMEOUT and its warp stops; nothing is computed or
@@ -271,10 +289,20 @@ LBM_API int lbm_check(lbm_lattice *h, int32_t *flags);
  * items a second launch also tests the wait in the middle of an item: one
  * item forms and publishes its edge moments (scratch that the next step
  * recomputes) and waits for neighbours that never run; *flags is
- * LBM_STATUS_TIMEOUT only if both launches raised it.  Synchronises the
- * device.  Not for batch members.
+ * LBM_STATUS_TIMEOUT only if both launches raised it.  For a lattice kept on
+ * the chip in two or more tiles it then runs lbm_selftest_resident_timeout's launch, if the
+ * inboxes can be allocated; again *flags is LBM_STATUS_TIMEOUT only if both raised it.
+ * Synchronises the device.  Not for batch members.
  */
 LBM_API int lbm_selftest_wait_timeout(lbm_lattice *h, int32_t *flags);
+
+/*
+ * The same of the waits of the launch that keeps a lattice on the chip, alone: every tile waits
+ * for values of a step that never runs (it allocates the inboxes as a first lbm_step would).  Returns
+ * LBM_ERR_INVALID_ARG for a lattice that the step kernel runs or of a single tile, and
+ * LBM_ERR_OOM without memory for the inboxes.
+ */
+LBM_API int lbm_selftest_resident_timeout(lbm_lattice *h, int32_t *flags);
 
 /*
  * Macroscopic fields at the current time: the Eq. 2 moments rho, u_x, u_r,
@@ -328,8 +356,8 @@ LBM_API int lbm_restore(lbm_lattice *h, const void *dev_in, int64_t step, lbm_st
  */
 LBM_API int lbm_set_launch(lbm_lattice *h, int32_t band_rows, int32_t warps_per_cta);
 
-/* The launch shape lbm_step uses: band height, warps per CTA and CTAs per
- * launch (any pointer may be NULL). */
+/* The launch shape of the step kernel: band height, warps per CTA and CTAs per
+ * launch (any pointer may be NULL).  Lattices kept on the chip: lbm_get_resident. */
 LBM_API int lbm_get_launch(const lbm_lattice *h, int32_t *band_rows, int32_t *warps_per_cta, int32_t *ctas);
 
 /* Work-item size of lbm_step's persistent launch: a warp takes `group`

@@ -304,6 +304,7 @@ struct lbm_lattice {
     size_t res_bytes;
     int64_t res_key;
     unsigned res_base;
+    int64_t res_steps;     // steps run by the resident launch since lbm_create
 
     void *buf(int b) const { return mem + L.off_buf[b]; }
     template <class T> T *at(size_t off) const { return reinterpret_cast<T *>(mem + off); }
@@ -576,12 +577,17 @@ lbm::ResCtl res_ctl(const lbm_lattice *h, const ResPlan &r, int nsteps)
     return ctl;
 }
 
+size_t res_bytes(const lbm_lattice *h, const ResPlan &r)
+{
+    return r.ns * r.nb < 2 ? 0 : (size_t)16 * (size_t)r.ns * (size_t)r.nb *
+                                     (size_t)lbm::res_box_words(h->d.storage == LBM_F64 ? 8 : 4, r.shape);
+}
+
 // The inboxes of the plan's tiles, ready for a launch on s.  *ok = false: there is no memory
 // for them, or none yet on a stream that is being captured.
 int res_ready(lbm_lattice *h, const ResPlan &r, bool capturing, cudaStream_t s, bool *ok)
 {
-    const size_t bytes = (size_t)16 * (size_t)r.ns * (size_t)r.nb *
-                         (size_t)lbm::res_box_words(h->d.storage == LBM_F64 ? 8 : 4, r.shape);
+    const size_t bytes = res_bytes(h, r);
     const int64_t key = ((int64_t)(r.shape + 1) << 40) | ((int64_t)r.ns << 20) | r.nb;
     *ok = r.ns * r.nb == 1;
     if (*ok)
@@ -639,6 +645,7 @@ int res_step(lbm_lattice *h, const ResPlan &r, int nsteps, bool capturing, cudaS
     h->res_base += (unsigned)nsteps;
     h->cur ^= (nsteps & 1);
     h->step += nsteps;
+    h->res_steps += nsteps;
     h->prev_valid = true;
     *done = nsteps;
     return LBM_OK;
@@ -1138,6 +1145,7 @@ int lbm_create(const lbm_desc *d, void *dev_mem, size_t bytes, lbm_lattice **out
     h->res_bytes = 0;
     h->res_key = 0;
     h->res_base = 0;
+    h->res_steps = 0;
     cudaGetDevice(&h->device);
     h->sms = 1;
     cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
@@ -1374,6 +1382,32 @@ static int step_impl(lbm_lattice *h, int32_t nsteps, lbm_stream stream)
     return LBM_OK;
 }
 
+// The resident launch, every tile starting at its second step and waiting for first steps that
+// never run.  *ran = false: no memory for the inboxes, or the tiles cannot all be resident.
+static int selftest_resident(lbm_lattice *h, int32_t *flags, bool *ran)
+{
+    const ResPlan r = h->res;
+    *ran = false;
+    if (r.shape < 0 || r.ns * r.nb < 2)
+        return LBM_OK;
+    bool ok = false;
+    int rc = res_ready(h, r, false, nullptr, &ok);
+    if (rc || !ok)
+        return rc;
+    lbm::ResCtl res = res_ctl(h, r, 2);
+    res.spin_limit = 64;
+    res.first = 1;
+    const cudaError_t e = res_launch(h, res, r, nullptr);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return LBM_OK;
+    }
+    if (e != cudaSuccess)
+        return cuda_fail(e, "self-test launch");
+    *ran = true;
+    return lbm_check(h, flags);
+}
+
 int lbm_selftest_wait_timeout(lbm_lattice *h, int32_t *flags)
 {
     if (!valid(h) || !flags)
@@ -1456,25 +1490,52 @@ int lbm_selftest_wait_timeout(lbm_lattice *h, int32_t *flags)
     if (e != cudaSuccess)
         return cuda_fail(e, "self-test launch");
     rc = lbm_check(h, flags);  // synchronises, reads and clears the status
-    const ResPlan r = h->res;
-    if (rc || r.shape < 0 || r.ns * r.nb < 2)
-        return rc;
-    // the resident launch: every tile starts at its second step and waits for first steps
-    // that never run
-    bool ok = false;
-    rc = res_ready(h, r, false, s, &ok);
-    if (rc || !ok)
-        return rc;
-    lbm::ResCtl res = res_ctl(h, r, 2);
-    res.spin_limit = 64;
-    res.first = 1;
-    e = res_launch(h, res, r, s);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "self-test launch");
     int32_t second = 0;
-    rc = lbm_check(h, &second);
-    *flags &= second;  // LBM_STATUS_TIMEOUT only if both launches' waits gave up
+    bool ran = false;
+    if (!rc)
+        rc = selftest_resident(h, &second, &ran);
+    if (ran)
+        *flags &= second;  // LBM_STATUS_TIMEOUT only if both launches' waits gave up
     return rc;
+}
+
+int lbm_selftest_resident_timeout(lbm_lattice *h, int32_t *flags)
+{
+    if (!valid(h) || !flags)
+        return fail(LBM_ERR_INVALID_ARG, "bad handle or NULL output");
+    if (h->batch || h->res.shape < 0 || h->res.ns * h->res.nb < 2)
+        return fail(LBM_ERR_INVALID_ARG, "the lattice has no tiles on the chip that wait for one another");
+    int32_t before = 0, v = 0;
+    bool ran = false;
+    int rc = lbm_check(h, &before);  // start from a clear status
+    if (!rc)
+        rc = selftest_resident(h, &v, &ran);
+    if (!rc && !ran)
+        rc = fail(LBM_ERR_OOM, "no memory for the inboxes, or the tiles cannot all be resident");
+    if (!rc)
+        *flags = v;
+    return rc;
+}
+
+int lbm_get_resident(const lbm_lattice *h, lbm_resident *out)
+{
+    if (!valid(h) || !out)
+        return fail(LBM_ERR_INVALID_ARG, "bad handle or NULL output");
+    const ResPlan &r = h->res;
+    const bool on = r.shape >= 0 && !h->batch;
+    std::memset(out, 0, sizeof(*out));
+    if (on) {
+        out->tile_cols = 32 * lbm::res_nv(r.shape, default_nv(h->d.storage));
+        out->tile_rows = lbm::res_rows(r.shape);
+        out->rows_per_warp = lbm::res_rpw(r.shape);
+        out->tiles_across = r.ns;
+        out->tiles_up = r.nb;
+        out->min_steps = res_min_steps(h->d.storage);
+        out->inbox_bytes = (int64_t)res_bytes(h, r);
+    }
+    out->inbox_held = (int64_t)h->res_bytes;
+    out->steps = h->res_steps;
+    return LBM_OK;
 }
 
 int lbm_set_item_group(lbm_lattice *h, int32_t group)

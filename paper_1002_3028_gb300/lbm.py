@@ -61,6 +61,14 @@ class Diag(C.Structure):
         return {name: getattr(self, name) for name, _ in self._fields_}
 
 
+class Resident(C.Structure):
+    """Mirror of ``lbm_resident``."""
+
+    _fields_ = [("tile_cols", C.c_int32), ("tile_rows", C.c_int32), ("rows_per_warp", C.c_int32),
+                ("tiles_across", C.c_int32), ("tiles_up", C.c_int32), ("min_steps", C.c_int32),
+                ("inbox_bytes", C.c_int64), ("inbox_held", C.c_int64), ("steps", C.c_int64)]
+
+
 def make_desc(cfg: LatticeConfig, storage: str, pattern: str = "ab") -> Desc:
     return Desc(pattern=PATTERN[pattern], nx=cfg.nx, nr=cfg.nr, storage=STORAGE[storage], bc_in=_BC_IN[cfg.bc_in],
                 bc_out=_BC_OUT[cfg.bc_out], bc_top=_BC_TOP[cfg.bc_top],
@@ -112,6 +120,8 @@ def lib(build: bool = True):
             L.lbm_get_launch.argtypes = [vp, C.POINTER(i32), C.POINTER(i32), C.POINTER(i32)]
             L.lbm_set_item_group.argtypes = [vp, i32]
             L.lbm_selftest_wait_timeout.argtypes = [vp, C.POINTER(i32)]
+            L.lbm_selftest_resident_timeout.argtypes = [vp, C.POINTER(i32)]
+            L.lbm_get_resident.argtypes = [vp, C.POINTER(Resident)]
             L.lbm_get_item_group.restype = i32
             L.lbm_get_item_group.argtypes = [vp]
             L.lbm_check.argtypes = [vp, C.POINTER(i32)]
@@ -278,8 +288,21 @@ class Lattice:
     def item_group(self) -> int:
         return int(self._L.lbm_get_item_group(self._h))
 
+    def selftest_resident_timeout(self) -> int:
+        """The same of the launch that keeps the lattice on the chip."""
+        v = C.c_int32()
+        _check(self._L.lbm_selftest_resident_timeout(self._h, C.byref(v)), "lbm_selftest_resident_timeout")
+        return v.value
+
+    def resident(self) -> dict:
+        """How ``step`` keeps the lattice on the chip (``lbm_resident``; tile_cols 0: it does not),
+        the device memory that takes beside ``nbytes``, and the steps run there so far."""
+        r = Resident()
+        _check(self._L.lbm_get_resident(self._h, C.byref(r)), "lbm_get_resident")
+        return {name: getattr(r, name) for name, _ in Resident._fields_}
+
     def launch(self):
-        """(band rows, warps per CTA, CTAs) used by lbm_step."""
+        """(band rows, warps per CTA, CTAs) of the step kernel (on the chip: ``resident``)."""
         b, w, c = C.c_int32(), C.c_int32(), C.c_int32()
         _check(self._L.lbm_get_launch(self._h, C.byref(b), C.byref(w), C.byref(c)), "lbm_get_launch")
         return b.value, w.value, c.value
