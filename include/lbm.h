@@ -194,12 +194,15 @@ LBM_API int lbm_set_properties(lbm_lattice *h, const double *nu, const double *a
  * persistent launch of the fused kernel (more than one only when nsteps x
  * warp tiles exceeds 2^30): a warp tile of step t + 1 starts once the tiles
  * around it have finished step t.  The result is bit for bit that of nsteps
- * one-step calls.  A two-buffer lattice that fits the GPU's shared memory (about
- * 300 000 nodes) and has no periodic ends and no launch shape of its own
- * (lbm_set_launch, lbm_set_item_group, lbm_set_strip_width) runs two steps
- * or more in one cooperative launch that keeps it on the chip; the first one
- * allocates up to 10 MB of device memory from the stream's memory pool, kept
- * until lbm_destroy (without it the lattice runs as the others do).  Asynchronous; returns LBM_ERR_CUDA if a launch fails.  A
+ * one-step calls.  A two-buffer lattice that fits the GPU's shared memory (up to about
+ * 300 000 nodes, FP64 78 000, on 152 SMs) and has no periodic ends and no launch shape of its own
+ * (lbm_set_launch, lbm_set_item_group, lbm_set_strip_width) runs calls of two steps or more (FP64:
+ * six) in one cooperative launch that keeps it on the chip; the first one allocates up to 10 MB of
+ * device memory from the stream's memory pool, beside lbm_required_bytes, kept until lbm_destroy
+ * (without it the lattice runs as the others do; lbm_get_resident).  Asynchronous; returns
+ * LBM_ERR_CUDA if a launch fails.  As every call on a lattice it waits for the lattice's set-up, an
+ * event outside any graph: on a stream that is being captured it returns LBM_ERR_CUDA, takes no
+ * step, and the capture is lost.  A
  * wait that runs out (it cannot in a correct launch; it is bounded all the
  * same) raises LBM_STATUS_TIMEOUT (see lbm_check) and ends the launch early.
  */

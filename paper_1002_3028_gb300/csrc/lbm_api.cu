@@ -295,14 +295,11 @@ struct lbm_lattice {
     // (lbm::RunCtl): valid for sync_items work items; 0 = reset before the next launch
     int64_t sync_items;
     unsigned sync_cbase, sync_fbase;
-    bool sync_captured;    // a launch was captured into a graph: reset before every launch
-    ResPlan res;           // resident launch (lbm_resident.cuh): its tiles; shape -1: none
-    // the tiles' inboxes of the resident launch, allocated by its first
-    // launch: valid for tiles laid out as res_key (0 = reset before the next launch), with
-    // res_base the number of the next launch's first step
+    ResPlan res;           // resident launch (lbm_resident.cuh): its tiles, planned once; shape -1: none
+    // the tiles' inboxes, allocated by the first resident launch; res_valid: they hold steps up
+    // to res_base, the number of the next launch's first step (else they are reset before it)
     void *res_box;
-    size_t res_bytes;
-    int64_t res_key;
+    bool res_valid;
     unsigned res_base;
     int64_t res_steps;     // steps run by the resident launch since lbm_create
 
@@ -400,8 +397,6 @@ lbm::StepParams<float> params_f(const lbm_lattice *h)
 // warp tiles per work item of lbm_step: the set value, else 1
 int item_group(const lbm_lattice *h) { return h->group > 0 ? h->group : 1; }
 
-void res_plan(lbm_lattice *h);
-
 // Launch shape of the step kernel: a persistent grid of one-warp CTAs (by
 // default) working through strip x band tiles.  A tile of step t + 1 waits
 // for the tiles around it of step t, which precede it by one step's worth
@@ -455,7 +450,6 @@ int plan_launch(lbm_lattice *h)
     const int64_t ntiles = (int64_t)nstrips * ((h->d.nr + h->band_eff - 1) / h->band_eff);
     h->ctas_max = per_sm * std::max(1, h->sms);
     h->ctas = (int)std::min<int64_t>(h->ctas_max, (ntiles + h->warps - 1) / h->warps);
-    res_plan(h);
     return LBM_OK;
 }
 
@@ -471,7 +465,13 @@ int plan_launch(lbm_lattice *h)
 //   64 x 16, two rows a warp, two a SM     1024 x 256 FP32 6.0 (12.4)
 // FP64 is bound by its arithmetic: the tiles that spread it over the SMs best.  The step
 // kernel keeps lattices that do not fit, those with periodic ends or in the AA layout, and
-// those whose launch shape the caller has set.
+// those whose launch shape the caller has set.  A lattice is planned once: its inboxes fit its
+// tiles as long as it lives.
+bool on_chip(const lbm_lattice *h)
+{
+    return h->res.shape >= 0 && h->band == 0 && h->group == 0 && h->warps == 1 && h->nv == default_nv(h->d.storage);
+}
+
 cudaError_t res_occupancy(const lbm_lattice *h, int shape, int warps, int *per_sm)
 {
     switch (h->d.storage) {
@@ -488,8 +488,7 @@ void res_plan(lbm_lattice *h)
 {
     const lbm_desc &d = h->d;
     h->res.shape = -1;
-    if (h->aa || d.bc_in == LBM_IN_PERIODIC || h->band > 0 || h->group > 0 || h->warps != 1 ||
-        h->nv != default_nv(d.storage))
+    if (h->aa || d.bc_in == LBM_IN_PERIODIC)
         return;
     auto fits = [&](int shape, int nb) {
         const int W = 32 * lbm::res_nv(shape, default_nv(d.storage));
@@ -579,42 +578,32 @@ lbm::ResCtl res_ctl(const lbm_lattice *h, const ResPlan &r, int nsteps)
 
 size_t res_bytes(const lbm_lattice *h, const ResPlan &r)
 {
-    return r.ns * r.nb < 2 ? 0 : (size_t)16 * (size_t)r.ns * (size_t)r.nb *
+    return r.shape < 0 || r.ns * r.nb < 2 ? 0 : (size_t)16 * (size_t)r.ns * (size_t)r.nb *
                                      (size_t)lbm::res_box_words(h->d.storage == LBM_F64 ? 8 : 4, r.shape);
 }
 
 // The inboxes of the plan's tiles, ready for a launch on s.  *ok = false: there is no memory
-// for them, or none yet on a stream that is being captured.
-int res_ready(lbm_lattice *h, const ResPlan &r, bool capturing, cudaStream_t s, bool *ok)
+// for them.
+int res_ready(lbm_lattice *h, const ResPlan &r, cudaStream_t s, bool *ok)
 {
     const size_t bytes = res_bytes(h, r);
-    const int64_t key = ((int64_t)(r.shape + 1) << 40) | ((int64_t)r.ns << 20) | r.nb;
-    *ok = r.ns * r.nb == 1;
+    *ok = bytes == 0;  // a single tile
     if (*ok)
         return LBM_OK;
-    cudaError_t e = cudaSuccess;
-    if (h->res_bytes < bytes) {
-        if (capturing)
-            return LBM_OK;
-        if (h->res_box)
-            cudaFreeAsync(h->res_box, s);
-        h->res_box = nullptr;
-        h->res_bytes = 0;
-        h->res_key = 0;
+    if (!h->res_box) {
         const RelaxedCapture relaxed;
         if (cudaMallocAsync(&h->res_box, bytes, s) != cudaSuccess) {
             cudaGetLastError();
             h->res_box = nullptr;
             return LBM_OK;
         }
-        h->res_bytes = bytes;
     }
-    if (h->res_key != key || h->sync_captured) {
-        e = cudaMemsetAsync(h->res_box, 0, bytes, s);
-        h->res_key = e == cudaSuccess ? key : 0;
-        h->res_base = 0;
+    if (!h->res_valid) {
+        const cudaError_t e = cudaMemsetAsync(h->res_box, 0, bytes, s);
         if (e != cudaSuccess)
             return cuda_fail(e, "inbox reset");
+        h->res_valid = true;
+        h->res_base = 0;
     }
     *ok = true;
     return LBM_OK;
@@ -626,11 +615,11 @@ int res_ready(lbm_lattice *h, const ResPlan &r, bool capturing, cudaStream_t s, 
 int res_min_steps(int storage) { return storage == LBM_F64 ? 6 : 2; }
 
 // *done: steps taken (fewer than nsteps when the tiles cannot all be resident after all)
-int res_step(lbm_lattice *h, const ResPlan &r, int nsteps, bool capturing, cudaStream_t s, int *done)
+int res_step(lbm_lattice *h, const ResPlan &r, int nsteps, cudaStream_t s, int *done)
 {
     bool ok = false;
     *done = 0;
-    int rc = res_ready(h, r, capturing, s, &ok);
+    int rc = res_ready(h, r, s, &ok);
     if (rc || !ok)
         return rc;
     cudaError_t e = res_launch(h, res_ctl(h, r, nsteps), r, s);
@@ -639,7 +628,7 @@ int res_step(lbm_lattice *h, const ResPlan &r, int nsteps, bool capturing, cudaS
         return LBM_OK;
     }
     if (e != cudaSuccess) {
-        h->res_key = 0;
+        h->res_valid = false;
         return cuda_fail(e, "resident step kernel launch");
     }
     h->res_base += (unsigned)nsteps;
@@ -1139,11 +1128,9 @@ int lbm_create(const lbm_desc *d, void *dev_mem, size_t bytes, lbm_lattice **out
     h->nv = default_nv(d->storage);
     h->sync_items = 0;
     h->sync_cbase = h->sync_fbase = 0;
-    h->sync_captured = false;
     h->res.shape = -1;
     h->res_box = nullptr;
-    h->res_bytes = 0;
-    h->res_key = 0;
+    h->res_valid = false;
     h->res_base = 0;
     h->res_steps = 0;
     cudaGetDevice(&h->device);
@@ -1202,6 +1189,8 @@ int lbm_create(const lbm_desc *d, void *dev_mem, size_t bytes, lbm_lattice **out
     if (!rc) rc = upload_pair(h, L.off_al_d, L.off_al_f, &one, 1, s0, "table upload");
     if (!rc)
         rc = plan_launch(h);
+    if (!rc)
+        res_plan(h);
     if (!rc)
         rc = fill_ghosts(h, s0);
     if (!rc) {
@@ -1318,17 +1307,9 @@ static int step_impl(lbm_lattice *h, int32_t nsteps, lbm_stream stream)
         }
         return LBM_OK;
     }
-    // The counters of either launch carry on from the previous launch (RunCtl, ResCtl) unless
-    // the tiles changed, a wait ran out (lbm_check) or the launch goes into a graph,
-    // whose replays must each start from a reset.
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess)
-        return cuda_fail(cudaGetLastError(), "querying the stream");
-    if (cap != cudaStreamCaptureStatusNone)
-        h->sync_captured = true;
-    if (nsteps >= res_min_steps(d.storage) && h->res.shape >= 0) {
+    if (nsteps >= res_min_steps(d.storage) && on_chip(h)) {
         int done = 0;
-        const int rc = res_step(h, h->res, nsteps, cap != cudaStreamCaptureStatusNone, s, &done);
+        const int rc = res_step(h, h->res, nsteps, s, &done);
         if (rc)
             return rc;
         nsteps -= done;
@@ -1343,10 +1324,12 @@ static int step_impl(lbm_lattice *h, int32_t nsteps, lbm_stream stream)
     ctl.radius = h->band_eff >= 2 ? 1 : 2;
     ctl.wrap = d.bc_in == LBM_IN_PERIODIC ? 1 : 0;
     ctl.spin_limit = lbm::RUN_SPIN_LIMIT;
+    // The counters carry on from the previous launch (RunCtl) unless the item count changed or a
+    // wait ran out (lbm_check).
     for (int64_t done = 0; done < nsteps;) {
         const int m = (int)std::min<int64_t>(per_launch, nsteps - done);
         cudaError_t e = cudaSuccess;
-        if (h->sync_items != items || h->sync_captured) {
+        if (h->sync_items != items) {
             e = cudaMemsetAsync(sync, 0, (size_t)4 * (size_t)(1 + items), s);
             if (e != cudaSuccess) {
                 h->sync_items = 0;
@@ -1388,10 +1371,10 @@ static int selftest_resident(lbm_lattice *h, int32_t *flags, bool *ran)
 {
     const ResPlan r = h->res;
     *ran = false;
-    if (r.shape < 0 || r.ns * r.nb < 2)
+    if (!on_chip(h) || r.ns * r.nb < 2)
         return LBM_OK;
     bool ok = false;
-    int rc = res_ready(h, r, false, nullptr, &ok);
+    int rc = res_ready(h, r, nullptr, &ok);
     if (rc || !ok)
         return rc;
     lbm::ResCtl res = res_ctl(h, r, 2);
@@ -1503,7 +1486,7 @@ int lbm_selftest_resident_timeout(lbm_lattice *h, int32_t *flags)
 {
     if (!valid(h) || !flags)
         return fail(LBM_ERR_INVALID_ARG, "bad handle or NULL output");
-    if (h->batch || h->res.shape < 0 || h->res.ns * h->res.nb < 2)
+    if (h->batch || !on_chip(h) || h->res.ns * h->res.nb < 2)
         return fail(LBM_ERR_INVALID_ARG, "the lattice has no tiles on the chip that wait for one another");
     int32_t before = 0, v = 0;
     bool ran = false;
@@ -1522,9 +1505,8 @@ int lbm_get_resident(const lbm_lattice *h, lbm_resident *out)
     if (!valid(h) || !out)
         return fail(LBM_ERR_INVALID_ARG, "bad handle or NULL output");
     const ResPlan &r = h->res;
-    const bool on = r.shape >= 0 && !h->batch;
     std::memset(out, 0, sizeof(*out));
-    if (on) {
+    if (on_chip(h) && !h->batch) {
         out->tile_cols = 32 * lbm::res_nv(r.shape, default_nv(h->d.storage));
         out->tile_rows = lbm::res_rows(r.shape);
         out->rows_per_warp = lbm::res_rpw(r.shape);
@@ -1533,7 +1515,7 @@ int lbm_get_resident(const lbm_lattice *h, lbm_resident *out)
         out->min_steps = res_min_steps(h->d.storage);
         out->inbox_bytes = (int64_t)res_bytes(h, r);
     }
-    out->inbox_held = (int64_t)h->res_bytes;
+    out->inbox_held = h->res_box ? (int64_t)res_bytes(h, h->res) : 0;
     out->steps = h->res_steps;
     return LBM_OK;
 }
@@ -1543,7 +1525,6 @@ int lbm_set_item_group(lbm_lattice *h, int32_t group)
     if (!valid(h) || group < 0 || group > 64)
         return fail(LBM_ERR_INVALID_ARG, "bad handle or group (0..64)");
     h->group = group;
-    res_plan(h);
     return LBM_OK;
 }
 
@@ -1591,8 +1572,10 @@ int lbm_check(lbm_lattice *h, int32_t *flags)
         e = cudaMemset(h->mem + h->L.off_status, 0, sizeof(int));
     if (e != cudaSuccess)
         return cuda_fail(e, "reading the status word");
-    if (v & lbm::STATUS_TIMEOUT)
-        h->sync_items = h->res_key = 0;  // a launch stopped early: its counters are not where the host expects
+    if (v & lbm::STATUS_TIMEOUT) {  // a launch stopped early: its counters are not where the host expects
+        h->sync_items = 0;
+        h->res_valid = false;
+    }
     *flags = v;
     return LBM_OK;
 }
