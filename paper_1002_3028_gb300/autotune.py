@@ -5,8 +5,10 @@ its stream (after a warm-up), three runs each, keeps the one whose slowest
 run is fastest, and remembers it in a small
 JSON cache keyed by the GPU name, the storage type and the lattice shape(s),
 so a later lattice of the same kind starts from the tuned shape.  The key
-also holds the memory pattern: the in-place (AA) kernel takes other strip
-widths and bands than the two-buffer one.  The tile
+also holds what else decides which shape is fastest: the memory pattern (the
+in-place (AA) kernel takes other strip widths and bands than the two-buffer
+one), which lattices have periodic ends (they never run on the chip), and the
+kernels' sources (a shape tuned for other code is not applied).  The tile
 is the warp's strip of 32 or 64 columns (one or two nodes per lane) by the
 band height; results are bit for bit the same for every shape.  Tuning steps
 the lattice: tune before setting the initial state, or save and restore it
@@ -14,6 +16,7 @@ the lattice: tune before setting the initial state, or save and restore it
 """
 from __future__ import annotations
 
+import functools
 import hashlib
 import json
 import os
@@ -28,7 +31,9 @@ CACHE = os.path.join(_build.BUILD, "autotune.json")
 # double the tiles of small lattices.  A batch spreads each step over many lattices and
 # profits from longer bands.
 LATTICE_CANDIDATES: Tuple[Tuple[int, int, int], ...] = (
-    (64, 0, 1), (32, 0, 1),  # band 0: the library's own choice, which keeps small lattices on the chip
+    # band 0: the library's own choice of band; with the storage type's own width (64 columns, FP64
+    # 32) it keeps lattices that fit on the chip
+    (64, 0, 1), (32, 0, 1),
     (64, 1, 1), (64, 2, 1), (64, 3, 1), (64, 4, 1), (64, 5, 1), (64, 6, 1), (64, 7, 1), (64, 8, 1), (64, 9, 1),
     (64, 10, 1), (64, 6, 2), (32, 1, 1), (32, 2, 1), (32, 4, 1), (32, 6, 1), (32, 8, 1),
 )
@@ -64,10 +69,21 @@ def _store(key: str, value) -> None:
         os.replace(tmp, CACHE)
 
 
-def lattice_key(storage: str, shapes: Iterable[Tuple[int, int]], pattern: str = "ab") -> str:
-    shapes = sorted(shapes)
+@functools.lru_cache(maxsize=None)
+def _code() -> str:
+    """Digest of the kernels' sources."""
+    h = hashlib.sha1()
+    for name in sorted(os.listdir(_build.CSRC)):
+        with open(os.path.join(_build.CSRC, name), "rb") as fh:
+            h.update(name.encode() + b"\0" + fh.read())
+    return h.hexdigest()[:12]
+
+
+def lattice_key(storage: str, shapes: Iterable[Tuple], pattern: str = "ab") -> str:
+    """shapes: (nx, nr) of every lattice, or (nx, nr, whether its axial ends are periodic)."""
+    shapes = sorted((s[0], s[1], bool(s[2]) if len(s) > 2 else False) for s in shapes)
     digest = hashlib.sha1(repr(shapes).encode()).hexdigest()[:12]
-    return f"{_gpu_name()}|{storage}|{pattern}|{len(shapes)}|{digest}"
+    return f"{_gpu_name()}|{storage}|{pattern}|{len(shapes)}|{digest}|{_code()}"
 
 
 def _time(step_fn, steps: int, warmup: int) -> float:
@@ -101,8 +117,8 @@ def tune(target, candidates: Optional[Sequence[Tuple[int, int, int]]] = None, st
     """Pick and set the fastest (strip columns, band rows, warps per CTA) for a Lattice or Batch.
 
     Returns the chosen shape.  With use_cache, a shape tuned earlier for the
-    same GPU, storage type, memory pattern and lattice shapes is applied
-    without timing.  Each
+    same GPU, storage type, memory pattern, lattice shapes and ends, and the
+    same kernels is applied without timing.  Each
     candidate runs `steps` steps in one persistent launch (enough that the
     launch's ramp and tail do not decide the ranking), three times, and is
     ranked by its slowest run.  Candidates with a strip width the lattice
@@ -112,7 +128,7 @@ def tune(target, candidates: Optional[Sequence[Tuple[int, int, int]]] = None, st
 
     is_batch = isinstance(target, Batch)
     members = target.members if is_batch else [target]
-    shapes = [(m.nx, m.nr) for m in members]
+    shapes = [(m.nx, m.nr, getattr(getattr(m, "cfg", None), "bc_in", "inlet") == "periodic") for m in members]
     pattern = members[0].pattern if members else "ab"
     key = lattice_key(target.storage, shapes, pattern)
     if use_cache:
