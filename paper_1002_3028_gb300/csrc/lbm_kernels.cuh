@@ -190,7 +190,6 @@ __device__ __forceinline__ const float *split_m(const S *buf, int64_t plane)
     return reinterpret_cast<const float *>(reinterpret_cast<const char *>(buf) + split_moff(plane));
 }
 
-// linear part of population q (deviation from rest) at moments (jx, jr, dT)
 // e.j for a lattice velocity e with components in {-1, 0, 1} (no product with a zero component)
 template <class C>
 __device__ __forceinline__ C edot(int ex, int ey, C jx, C jr)
@@ -199,6 +198,7 @@ __device__ __forceinline__ C edot(int ex, int ey, C jx, C jr)
     return ex == 0 ? (ey == 0 ? C(0) : b) : (ey == 0 ? a : a + b);
 }
 
+// linear part of population q (deviation from rest) at moments (jx, jr, dT)
 template <class C>
 __device__ __forceinline__ C lin_part(const StepParams<C> &p, int q, C jx, C jr, C dT)
 {
@@ -211,14 +211,16 @@ __device__ __forceinline__ C lin_part(const StepParams<C> &p, int q, C jx, C jr,
 
 // A population from its stored deviation d and the moments stored with it (the linear part
 // added), and the deviation of a population v at moments (jx, jr, dT) (the linear part taken
-// off), with the roundings of stage_pops and of collide_row's store: for the kernels whose
-// values must have the step kernel's bits without its surroundings (rn_*: below).
+// off).  Their roundings are fixed (rn_*: below), not left to the compiler's contraction: every
+// kernel that advances a lattice has to give the same bits.
 template <class C> __device__ __forceinline__ C split_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d);
 template <class C> __device__ __forceinline__ C split_sub(const StepParams<C> &p, int q, C jx, C jr, C dT, C v);
-// The same with the roundings of write_ghosts: an edge node's populations from what it
+// The same with the roundings of the ghost rules: an edge node's populations from what it
 // stored (a state read out has these too), and what its ghost cells store.
 template <class C> __device__ __forceinline__ C edge_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d);
 template <class C> __device__ __forceinline__ C edge_sub(const StepParams<C> &p, int q, C jx, C jr, C dT, C v);
+// ... and with those of a single node's pull, for the fields and the diagnostics.
+template <class C> __device__ __forceinline__ C pull_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d);
 
 // Moments a ghost cell (ci, cj) carries when node (i, j), with moments
 // (jx, jr, dT), writes it: the one node whose rule fills an axis, open-top,
@@ -329,6 +331,15 @@ __device__ __forceinline__ C edge_sub(const StepParams<C> &p, int q, C jx, C jr,
         return split_sub<C>(p, q, jx, jr, dT, v);
     const C x = rn_mul(rn_add(p.T0, dT), p.hir0);
     return rn_sub(v, rn_fma(C(0.25), dT, rn_mul(x, edot<C>(ex4(q - 9), ey4(q - 9), jx, jr))));
+}
+
+template <class C>
+__device__ __forceinline__ C pull_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d)
+{
+    if (q < 9)
+        return split_add<C>(p, q, jx, jr, dT, d);
+    const C x = rn_mul(rn_add(p.T0, dT), p.hir0);
+    return rn_add(d, rn_fma(C(0.25), dT, rn_mul(x, edot<C>(ex4(q - 9), ey4(q - 9), jx, jr))));
 }
 
 template <class C> __device__ __forceinline__ Vec<C, 1> operator+(Vec<C, 1> a, Vec<C, 1> b) { return Vec<C, 1>(rn_add(a.x, b.x)); }
@@ -608,10 +619,10 @@ __device__ __noinline__ void write_ghosts(const StepParams<C> &p, S *buf, int i,
         const C jx = jj.x, jr = jj.y, dT = M.T(o);
 #pragma unroll
         for (int k = 0; k < 9; ++k)
-            fo[k] = lin_part<C>(p, k, jx, jr, dT) + load_as_shared<S, C>(buf + cell(p, k, i, j));
+            fo[k] = edge_add<C>(p, k, jx, jr, dT, load_as_shared<S, C>(buf + cell(p, k, i, j)));
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            go[k] = lin_part<C>(p, 9 + k, jx, jr, dT) + load_as_shared<S, C>(buf + cell(p, 9 + k, i, j));
+            go[k] = edge_add<C>(p, 9 + k, jx, jr, dT, load_as_shared<S, C>(buf + cell(p, 9 + k, i, j)));
         ghost_rules<C>(p, fo, go, i, j, t, [&](int q, int ci, int cj, C v) {
             C gx, gr, gT;
             const int64_t oc = cell(p, 0, ci, cj);
@@ -619,7 +630,8 @@ __device__ __noinline__ void write_ghosts(const StepParams<C> &p, S *buf, int i,
                                  [&]() -> C { return p.T_in[cj]; }, gx, gr, gT)) {
                 M.j(oc) = make_float2(gx, gr);
                 M.T(oc) = gT;
-                v -= lin_part<C>(p, q, gx, gr, gT);
+                // (beyond the axis, whose is the one g1 with moments, as in a collision's store)
+                v = q == 10 ? split_sub<C>(p, q, gx, gr, gT, v) : edge_sub<C>(p, q, gx, gr, gT, v);
             }
             buf[cell(p, q, ci, cj)] = store_as<S, C>(v);
         });
@@ -656,7 +668,7 @@ __device__ __forceinline__ C pulled(const StepParams<C> &p, const S *src, int q,
         const float *M = split_m(src, p.plane);
         const int64_t o = c - (int64_t)q * p.plane;
         const float2 jj = __ldcg(reinterpret_cast<const float2 *>(M) + o);
-        v += lin_part<C>(p, q, jj.x, jj.y, __ldcg(M + 2 * p.plane + o));
+        v = pull_add<C>(p, q, jj.x, jj.y, __ldcg(M + 2 * p.plane + o), v);
     }
     return v;
 }
@@ -1113,7 +1125,7 @@ __device__ __forceinline__ C spop(const StepParams<C> &p, const S *stage, const 
     C v = sget<S, NV, C>(stage, q, ex, lane + off);
     if constexpr (IsSplit<S>::value) {
         const float2 jj = mr.j[1 - ey][off - ex];
-        v += lin_part<C>(p, q, jj.x, jj.y, q < 9 ? C(0) : mr.T[1 - ey][off - ex]);
+        v = split_add<C>(p, q, jj.x, jj.y, q < 9 ? C(0) : mr.T[1 - ey][off - ex], v);
     }
     return v;
 }
@@ -1252,10 +1264,10 @@ __device__ __forceinline__ void collide_row(const StepParams<C> &p, const S *src
                 M.T(o) = dT;
 #pragma unroll
                 for (int k = 0; k < 9; ++k)
-                    dst[o + k * pl] = store_as<S, C>(fo[k][c] - lin_part<C>(p, k, jx, jr, dT));
+                    dst[o + k * pl] = store_as<S, C>(split_sub<C>(p, k, jx, jr, dT, fo[k][c]));
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    dst[o + (9 + k) * pl] = store_as<S, C>(go[k][c] - lin_part<C>(p, 9 + k, jx, jr, dT));
+                    dst[o + (9 + k) * pl] = store_as<S, C>(split_sub<C>(p, 9 + k, jx, jr, dT, go[k][c]));
             } else {
 #pragma unroll
                 for (int k = 0; k < 9; ++k)

@@ -175,15 +175,6 @@ __device__ __forceinline__ void put_field(double *o, float v)
     *o = (__float_as_uint(v) << 1) == 0 ? __hiloint2double((int)__float_as_uint(v), 0) : diag_double(v);
 }
 
-// moment-split storage: a thermal population from its deviation, as the linear part's sum rounds
-// when it is formed before the deviation is added
-template <class C>
-__device__ __forceinline__ C field_add(const StepParams<C> &p, int q, C jx, C jr, C dT, C d)
-{
-    const C x = rn_mul(rn_add(p.T0, dT), p.hir0);
-    return rn_add(d, rn_fma(C(0.25), dT, rn_mul(x, edot<C>(ex4(q - 9), ey4(q - 9), jx, jr))));
-}
-
 // A node a lane, all of its loads in flight together; a CTA takes 32 columns by eight rows, so
 // that the moments of moment-split storage, which the nodes of three rows read, come from L1.
 // Bound by memory in FP32.  4096 x 1024 into FP64 / FP32 fields, us, before (a node a thread in
@@ -233,7 +224,7 @@ __global__ void __launch_bounds__(256) fields_kernel(const __grid_constant__ Ste
                 f[q].x = edge_add<C>(p, q, jj[q].x, jj[q].y, 0.f, f[q].x);
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                g[q].x = field_add<C>(p, 9 + q, jj[q + 1].x, jj[q + 1].y, T[q], g[q].x);
+                g[q].x = pull_add<C>(p, 9 + q, jj[q + 1].x, jj[q + 1].y, T[q], g[q].x);
         }
         const Mom<Vec<C, 1>> m = moments<Vec<C, 1>>(f, g);
         const C rho = p.rho0 + m.drho.x;
