@@ -291,6 +291,7 @@ struct lbm_lattice {
     int phase;             // AA pattern: representation of the stored state (lbm_aa.cuh)
     cudaEvent_t ready;     // recorded after the set-up work lbm_create enqueued
     cudaEvent_t last;      // recorded after the last work enqueued on the lattice
+    cudaStream_t last_on;  // ... on this stream (which may be gone by now)
     // counters of the two-buffer persistent launch, carried from launch to launch
     // (lbm::RunCtl): valid for sync_items work items; 0 = reset before the next launch
     int64_t sync_items;
@@ -527,8 +528,47 @@ struct RelaxedCapture {
     ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
-// Releases the inboxes after the lattice's last use, on a stream that orders nothing else (the
-// default stream would hold up the caller's work on it until then).
+// The current device's stream for releases: non-blocking, made once and kept (making and
+// destroying one for each release took up to 80 us), and made again in a context that a device
+// reset has replaced (its id differs).  nullptr if it cannot be made.
+cudaStream_t release_stream()
+{
+    using GetId = int (*)(void *, unsigned long long *);
+    struct Kept {
+        cudaStream_t s;
+        unsigned long long context;
+    };
+    static std::mutex m;
+    static Kept kept[64] = {};
+    static GetId get_id = nullptr;
+    int device = -1;
+    if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64)
+        return nullptr;
+    std::lock_guard<std::mutex> lock(m);
+    if (!get_id) {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            return nullptr;
+        get_id = reinterpret_cast<GetId>(fn);
+    }
+    unsigned long long context = 0;
+    if (get_id(nullptr, &context) != 0)
+        return nullptr;
+    Kept &k = kept[device];
+    if (!k.s || k.context != context) {
+        k.context = context;
+        if (cudaStreamCreateWithFlags(&k.s, cudaStreamNonBlocking) != cudaSuccess)
+            k.s = nullptr;
+    }
+    return k.s;
+}
+
+// Releases the inboxes after the lattice's last use: on the default stream if that is where it
+// was (the next lattice there takes the memory over without a wait; a served request 2278 -> 2257
+// us), else on a stream that orders nothing else (the default stream would hold up the caller's
+// work on it until then).
 void res_release(lbm_lattice *h)
 {
     if (!h->res_box)
@@ -538,13 +578,9 @@ void res_release(lbm_lattice *h)
     cudaGetDevice(&device);
     if (device != h->device)
         cudaSetDevice(h->device);
-    cudaStream_t s = nullptr;
-    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess)
-        s = nullptr;
+    cudaStream_t s = h->last_on ? release_stream() : nullptr;
     cudaStreamWaitEvent(s, h->last, 0);
     cudaFreeAsync(h->res_box, s);
-    if (s)
-        cudaStreamDestroy(s);  // once its work has run
     if (device != h->device)
         cudaSetDevice(device);
     cudaGetLastError();
@@ -766,6 +802,7 @@ int leave(lbm_lattice *h, cudaStream_t s, int rc)
         cudaError_t e = cudaEventRecord(h->last, s);
         if (e != cudaSuccess)
             return cuda_fail(e, "recording the lattice's last use");
+        h->last_on = s;
     }
     return rc;
 }
@@ -1141,6 +1178,7 @@ int lbm_create(const lbm_desc *d, void *dev_mem, size_t bytes, lbm_lattice **out
     // `ready` event (enter), so creating a lattice never drains the device.
     cudaStream_t s0 = nullptr;
     h->ready = h->last = nullptr;
+    h->last_on = nullptr;
     cudaError_t e = cudaEventCreateWithFlags(&h->ready, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaEventCreateWithFlags(&h->last, cudaEventDisableTiming);

@@ -47,9 +47,11 @@ def test_inboxes_are_given_back(lbm):
     assert cycle(60) > free - 64 * 2 ** 20  # an inbox each would be 500 MB
 
 
-def test_a_first_step_leaves_another_streams_capture_alone(lbm):
+@pytest.mark.parametrize("default_stream", [False, True])
+def test_a_first_step_leaves_another_streams_capture_alone(lbm, default_stream):
     lat = lbm.Lattice.from_workload(I.jet_workload(nx=200, nr=96), "f32", device="cuda:0")
-    side, x = torch.cuda.Stream(), torch.zeros(8, device="cuda:0")
+    side = torch.cuda.default_stream() if default_stream else torch.cuda.Stream()
+    x = torch.zeros(8, device="cuda:0")
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, capture_error_mode="global"):
