@@ -199,7 +199,9 @@ LBM_API int lbm_set_properties(lbm_lattice *h, const double *nu, const double *a
  * (lbm_set_launch, lbm_set_item_group, lbm_set_strip_width) runs calls of two steps or more (FP64:
  * six) in one cooperative launch that keeps it on the chip; the first one allocates up to 10 MB of
  * device memory from the stream's memory pool, beside lbm_required_bytes, kept until lbm_destroy
- * (without it the lattice runs as the others do; lbm_get_resident).  Asynchronous; returns
+ * (without it the lattice runs as the others do; lbm_get_resident).  Lattices of fewer than 42 000
+ * nodes of which no two fit the chip together (not the moment-split types) take the step kernel
+ * while others of them run on three other streams (FP64: on one).  Asynchronous; returns
  * LBM_ERR_CUDA if a launch fails.  As every call on a lattice it waits for the lattice's set-up, an
  * event outside any graph: on a stream that is being captured it returns LBM_ERR_CUDA, takes no
  * step, and the capture is lost.  A
@@ -214,8 +216,8 @@ LBM_API int lbm_step(lbm_lattice *h, int32_t nsteps, lbm_stream stream);
  * all 0 for a lattice that the step kernel runs.  min_steps: the steps from which a call runs
  * there.  inbox_bytes: the device memory that the first such call allocates beside the memory of
  * lbm_required_bytes (0 for a single tile); inbox_held: what is allocated now.  steps: the steps
- * that have run there since lbm_create (fewer than were asked for where the inboxes could not
- * be allocated: the step kernel took those).
+ * that have run there since lbm_create (the step kernel took the others: calls of fewer steps,
+ * beside other streams' lattices, without memory for the inboxes).
  */
 typedef struct {
     int32_t tile_cols, tile_rows, rows_per_warp;

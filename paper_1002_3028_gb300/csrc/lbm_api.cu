@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -268,6 +269,7 @@ struct lbm_batch;
 
 struct ResPlan {  // tiles of a lattice kept on the chip (res_plan)
     int shape, ns, nb, warps;
+    bool alone;  // no second such lattice fits beside it
 };
 
 struct lbm_lattice {
@@ -291,7 +293,8 @@ struct lbm_lattice {
     int phase;             // AA pattern: representation of the stored state (lbm_aa.cuh)
     cudaEvent_t ready;     // recorded after the set-up work lbm_create enqueued
     cudaEvent_t last;      // recorded after the last work enqueued on the lattice
-    cudaStream_t last_on;  // ... on this stream (which may be gone by now)
+    std::atomic<cudaStream_t> last_on;  // ... on this stream (which may be gone by now)
+    bool flying;           // listed in flights(), whose mutex guards it
     // counters of the two-buffer persistent launch, carried from launch to launch
     // (lbm::RunCtl): valid for sync_items work items; 0 = reset before the next launch
     int64_t sync_items;
@@ -505,7 +508,7 @@ void res_plan(lbm_lattice *h)
         }
         if ((int64_t)ns * nb > (int64_t)per_sm * h->sms)
             return false;
-        h->res = ResPlan{shape, ns, nb, warps};
+        h->res = ResPlan{shape, ns, nb, warps, 2 * ns * nb > per_sm * h->sms};
         return true;
     };
     // tiles up when `slots` CTAs share the lattice in tiles of at least `rows` rows
@@ -578,7 +581,7 @@ void res_release(lbm_lattice *h)
     cudaGetDevice(&device);
     if (device != h->device)
         cudaSetDevice(h->device);
-    cudaStream_t s = h->last_on ? release_stream() : nullptr;
+    cudaStream_t s = h->last_on.load() ? release_stream() : nullptr;
     cudaStreamWaitEvent(s, h->last, 0);
     cudaFreeAsync(h->res_box, s);
     if (device != h->device)
@@ -643,6 +646,78 @@ int res_ready(lbm_lattice *h, const ResPlan &r, cudaStream_t s, bool *ok)
     }
     *ok = true;
     return LBM_OK;
+}
+
+// Several lattices on several streams.  Resident launches that take more than half of the chip
+// run one after the other, where the step kernel's CTAs of small lattices run side by side: from
+// some number of them on, the step kernel advances them all sooner.  us a step of all K lattices,
+// step kernel / resident / by this rule (five calls of 150 steps each; the first ones are resident):
+//   200 x 96 FP32     K = 3 10.6 / 8.9 / 8.9     K = 4 11.1 / 11.9 / 11.9   K = 10 18.5 / 29.6 / 18.3
+//   300 x 120 FP32    K = 3 11.3 / 8.9 / 9.0     K = 4 11.9 / 11.9 / 13.2   K = 10 29.1 / 29.7 / 29.0
+//   400 x 100 FP16    K = 3 11.4 / 10.4 / 10.4   K = 4 11.6 / 13.9 / 12.7   K = 10 29.6 / 34.7 / 29.4
+//   400 x 120 FP32    K = 4 16.2 / 13.7          K = 10 39.5 / 34.3         (larger ones win by more)
+//   200 x 96 FP64     K = 2 27.4 / 33.1 / 31.1   K = 10 125 / 162 / 126     (500 x 130: 375 / 355)
+//   400 x 100 FP64    K = 2 45.9 / 50.7 / 46.9   K = 10 228 / 254 / 229
+// and in moment-split storage the resident launches are never slower (200 x 96 K = 10 34.1 / 33.8).
+// So lattices of fewer than 42 000 nodes in the other types, two of which do not fit beside one
+// another, leave the chip to the step kernel while others of them are in flight on three other
+// streams, in FP64 on one.  Only which kernel runs depends on it, no result.
+bool res_yields(const lbm_lattice *h)
+{
+    return h->res.alone && !is_split(h->d.storage) && (int64_t)h->d.nx * h->d.nr < 42000;
+}
+
+// the lattices of this kind whose last call may still be running
+struct Flights {
+    std::mutex m;
+    std::vector<lbm_lattice *> v;
+};
+Flights &flights()
+{
+    static Flights *f = new Flights;  // (outlives the lattices that other static objects hold)
+    return *f;
+}
+
+bool res_crowded(const lbm_lattice *h, cudaStream_t s)
+{
+    const int limit = h->d.storage == LBM_F64 ? 1 : 3;
+    cudaStream_t seen[3];
+    int others = 0;  // streams with such a lattice in flight (those of one stream run in turn)
+    const RelaxedCapture relaxed;
+    Flights &f = flights();
+    std::lock_guard<std::mutex> lock(f.m);
+    for (size_t n = 0; n < f.v.size() && others < limit;) {
+        lbm_lattice *g = f.v[n];
+        if (g == h || g->device != h->device) {
+            ++n;
+            continue;
+        }
+        const cudaError_t e = cudaEventQuery(g->last);
+        if (e != cudaSuccess)
+            cudaGetLastError();
+        if (e == cudaErrorNotReady) {
+            const cudaStream_t on = g->last_on.load();
+            if (on != s && std::find(seen, seen + others, on) == seen + others)
+                seen[others++] = on;
+            ++n;
+        } else {
+            g->flying = false;
+            f.v[n] = f.v.back();
+            f.v.pop_back();
+        }
+    }
+    return others >= limit;
+}
+
+void flight_list(lbm_lattice *h, bool in)
+{
+    Flights &f = flights();
+    std::lock_guard<std::mutex> lock(f.m);
+    if (in && !h->flying)
+        f.v.push_back(h);
+    if (!in && h->flying)
+        f.v.erase(std::find(f.v.begin(), f.v.end(), h));
+    h->flying = in;
 }
 
 // steps from which a call is worth the load of the tiles and their rings (us for 2 steps, the
@@ -1179,6 +1254,7 @@ int lbm_create(const lbm_desc *d, void *dev_mem, size_t bytes, lbm_lattice **out
     cudaStream_t s0 = nullptr;
     h->ready = h->last = nullptr;
     h->last_on = nullptr;
+    h->flying = false;
     cudaError_t e = cudaEventCreateWithFlags(&h->ready, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaEventCreateWithFlags(&h->last, cudaEventDisableTiming);
@@ -1252,6 +1328,7 @@ void lbm_destroy(lbm_lattice *h)
         return;
     if (h->batch)
         lbm_batch_remove(h->batch, h);
+    flight_list(h, false);
     if (h->own && h->mem) {
         // released in stream order after the lattice's last use: no host synchronisation
         cudaStreamWaitEvent(nullptr, h->last, 0);
@@ -1345,7 +1422,7 @@ static int step_impl(lbm_lattice *h, int32_t nsteps, lbm_stream stream)
         }
         return LBM_OK;
     }
-    if (nsteps >= res_min_steps(d.storage) && on_chip(h)) {
+    if (nsteps >= res_min_steps(d.storage) && on_chip(h) && !(res_yields(h) && res_crowded(h, s))) {
         int done = 0;
         const int rc = res_step(h, h->res, nsteps, s, &done);
         if (rc)
@@ -2025,7 +2102,12 @@ int lbm_step(lbm_lattice *h, int32_t nsteps, lbm_stream stream)
         return fail(LBM_ERR_INVALID_ARG, "bad lattice handle");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int rc = enter(h, s);
-    return rc ? rc : leave(h, s, step_impl(h, nsteps, stream));
+    if (rc)
+        return rc;
+    const int done = leave(h, s, step_impl(h, nsteps, stream));
+    if (done == LBM_OK && res_yields(h))
+        flight_list(h, true);
+    return done;
 }
 
 int lbm_get_fields(lbm_lattice *h, void *dev_out, int32_t out_type, lbm_stream stream)
