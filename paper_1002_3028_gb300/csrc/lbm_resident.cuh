@@ -292,11 +292,13 @@ __device__ __noinline__ void res_lists(const StepParams<C> &p, const int ns, con
 
 // ---- receiving ---------------------------------------------------------------------------
 // one more poll of a wait?  Sleeps between polls; false, in the whole warp, when the wait runs out or
-// another's did.
+// another's did.  (A vote; with lane 0's reading handed round, as in wait_given_up, a step took 1%
+// longer here.)
 template <class C>
 __device__ __forceinline__ bool res_poll_again(const StepParams<C> &p, int spin_limit, int it)
 {
-    if (it >= spin_limit || (it > 64 && wait_given_up(p.status)))
+    if (it >= spin_limit ||
+        (it > 64 && __any_sync(0xffffffffu, *static_cast<const volatile int *>(p.status) & STATUS_TIMEOUT)))
         return false;
     if (it > 32)
         __nanosleep(it < 256 ? 32 : 1024);
