@@ -19,10 +19,10 @@
 // of one tile through L2: staged rows, moments, one collision, stores, the
 // release and the neighbours' acquire.  Here a step is two barriers, one
 // collision's latency per row a warp holds, and the exchange of the ring.
-// us per step, the step kernel against this one (200 steps a launch):
-// 64 x 32 FP32 6.6 -> 3.0, 200 x 96 FP32 8.6 -> 3.0 and FP64 19.4 -> 16.1,
-// 900 x 140 FP32 11.5 -> 4.4, 640 x 160 FP16 moment-split 15.2 -> 4.4,
-// 1024 x 256 16.2 -> 7.3 and FP32 12.5 -> 6.0.  With the exchange's waits taken out the last
+// us per step, the step kernel against this one (one jet, 200 steps a launch):
+// 64 x 32 FP32 6.7 -> 3.0 (the pipe 5.2 -> 2.9), 200 x 96 FP32 8.7 -> 3.0 and FP64 19.5 -> 16.1,
+// 900 x 140 FP32 11.5 -> 4.3, 640 x 160 FP16 moment-split 15.4 -> 4.4,
+// 1024 x 256 16.4 -> 7.3 and FP32 12.6 -> 6.0.  With the exchange's waits taken out the last
 // takes 4.6: the rest is the way of a value through L2 and the slowest tile
 // of each neighbourhood, one at a lattice edge, whose ghosts come after its
 // collisions.
