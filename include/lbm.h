@@ -61,7 +61,7 @@ typedef enum {
     LBM_ERR_INVALID_ARG = -1, /* bad handle, size, boundary kind or table */
     LBM_ERR_OOM = -2,         /* device allocation failed or caller memory too small */
     LBM_ERR_CUDA = -3,        /* a CUDA runtime call or a kernel launch failed */
-    LBM_ERR_DIVERGED = -4     /* non-finite or non-positive density / temperature found */
+    LBM_ERR_DIVERGED = -4     /* non-finite or non-positive density, or non-finite velocity or temperature, found */
 } lbm_status;
 
 /* storage type of the populations on the device (the arithmetic is FP64
