@@ -1159,7 +1159,8 @@ int finish_diag(const double *v, int have_prev, lbm_diag *out)
     out->residual_max = (have_prev && v[6] > 0.0) ? std::sqrt(v[5]) / std::sqrt(v[6]) : nan;
     out->nonfinite = (int64_t)v[7];
     if (out->nonfinite > 0)
-        return fail(LBM_ERR_DIVERGED, "%lld nodes with a non-finite or non-positive density or a non-finite velocity or temperature",
+        return fail(LBM_ERR_DIVERGED,
+                    "%lld nodes with a non-finite or non-positive density or a non-finite velocity or temperature",
                     (long long)out->nonfinite);
     return LBM_OK;
 }
